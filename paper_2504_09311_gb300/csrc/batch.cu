@@ -739,8 +739,6 @@ static int peel_large_concurrent(dupin_graph *const *graphs, const dupin_params 
             rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_BULK, s, nullptr,
                                      grid > 0 ? grid : 1);
             if (rc) break;
-            // the later peels' grid-wide rounds run narrow beside this one's tail if it is a cluster
-            for (size_t q2 = q + 1; q2 < k; q2++) enqueue_note_cluster(ws[q], ws[q2], s);
         }
         rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_BUILD, s);
         if (rc) break;
@@ -760,6 +758,39 @@ static int peel_large_concurrent(dupin_graph *const *graphs, const dupin_params 
         rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_TAIL, t);
         if (rc) break;
         held += plans[q].cl_cap > 0 ? cl_sms : 1;
+        e = cudaEventRecord(ev[2 * q + 1], t);
+        if (e != cudaSuccess) rc = dupin_cuda_fail(e, "tail stream join");
+    }
+    // A peel that its cluster tail gave back runs its grid-wide rounds again on
+    // 's' (one cooperative launch at a time), on the SMs that no other peel's
+    // tail may hold, and its tails again on its own stream; with many peels,
+    // one after another once every tail is done.
+    for (size_t q = 0; q < k && rc == DUPIN_OK && !overlap; q++) {
+        cudaError_t e = cudaStreamWaitEvent(s, ev[2 * q + 1], 0);
+        if (e != cudaSuccess) rc = dupin_cuda_fail(e, "tail stream join");
+    }
+    for (size_t q = 0; q < k && rc == DUPIN_OK; q++) {
+        if (!peel_again(graphs[idx[q]], &params[idx[q]], plans[q])) continue;
+        if (!overlap) {
+            rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_BULK2 | PEEL_TAIL2, s);
+            continue;
+        }
+        cudaStream_t t = tail_stream(dev, q);
+        cudaError_t e = cudaStreamWaitEvent(s, ev[2 * q + 1], 0);
+        if (e == cudaSuccess) {
+            const int grid = ws[q]->grid - (held - (plans[q].cl_cap > 0 ? cl_sms : 1));
+            rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_BULK2, s, nullptr,
+                                     grid > 0 ? grid : 1);
+            if (rc) break;
+            e = cudaEventRecord(ev[2 * q], s);
+        }
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(t, ev[2 * q], 0);
+        if (e != cudaSuccess) {
+            rc = dupin_cuda_fail(e, "tail stream setup");
+            break;
+        }
+        rc = enqueue_peel_stages(graphs[idx[q]], ws[q], &params[idx[q]], plans[q], PEEL_TAIL2, t);
+        if (rc) break;
         e = cudaEventRecord(ev[2 * q + 1], t);
         if (e != cudaSuccess) rc = dupin_cuda_fail(e, "tail stream join");
     }

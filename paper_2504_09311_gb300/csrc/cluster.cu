@@ -57,6 +57,7 @@
 #include <mutex>
 #include <string>
 
+#include "cluster_device.cuh"
 #include "dupin_internal.h"
 #include "peel_device.cuh"
 
@@ -69,40 +70,6 @@
 #define CL_ILP 4    // arcs in flight per thread in the expand
 #define CL_MAXC 16
 static const long long kPad = (long long)0x8000000000000000ULL;  // slots past the owned ones
-
-// ------------------------------------------------------------- cluster PTX
-
-__device__ __forceinline__ unsigned cl_rank() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ unsigned cl_size() {
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
-// all threads of every CTA of the cluster; release/acquire orders the
-// shared-memory writes (local and remote) before it against reads after it
-__device__ __forceinline__ void cl_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// the shared::cluster address of 'p' (this CTA's shared memory) in CTA 'rank'
-__device__ __forceinline__ uint32_t cl_map(const void *p, unsigned rank) {
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    uint32_t o;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(rank));
-    return o;
-}
-
-__device__ __forceinline__ unsigned cl_ld_u16(uint32_t a) {
-    unsigned short v;
-    asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
-    return v;
-}
 
 // ------------------------------------------------------------ shared state
 
@@ -160,63 +127,6 @@ __device__ __forceinline__ long long block_min64(long long x, long long *s) {
     long long m = lane < CL_WARPS ? s[lane] : kMaxLL;
     m = warp_min64(m);
     return m;
-}
-
-__device__ __forceinline__ void cl_st_u32(uint32_t a, unsigned x) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
-}
-
-// 16 bytes into another CTA's shared memory, completing (as 16 transaction
-// bytes) on the mbarrier at 'mbar' in that CTA
-__device__ __forceinline__ void cl_st_async_v4(uint32_t a, uint32_t mbar, unsigned x, unsigned y, unsigned z,
-                                               unsigned w) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
-                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mb_init(unsigned long long *mb, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(mb)), "r"(count)
-                 : "memory");
-}
-
-// this thread's arrival, announcing 'tx' transaction bytes for the current phase
-__device__ __forceinline__ void mb_arrive_expect_tx(unsigned long long *mb, unsigned tx) {
-    asm volatile(
-        "{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(
-            (unsigned)__cvta_generic_to_shared(mb)),
-        "r"(tx)
-        : "memory");
-}
-
-// has the phase of parity 'parity' completed? (acquire at cluster scope: the
-// asynchronous stores that completed it are visible)
-__device__ __forceinline__ bool mb_try_wait(unsigned long long *mb, unsigned parity) {
-    unsigned done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, "
-        "1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"((unsigned)__cvta_generic_to_shared(mb)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
-__device__ __forceinline__ void cl_st_u64(uint32_t a, unsigned long long x) {
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(x) : "memory");
-}
-
-// L2 prefetch of bytes [off, off + len) of an array of 'total' bytes, in
-// 16-byte granules inside the array (one bulk request, no data returned)
-__device__ __forceinline__ void prefetch_l2(const void *base, unsigned long long total, unsigned long long off,
-                                            unsigned long long len) {
-    const unsigned long long a = off & ~15ull;
-    unsigned long long b = (off + len + 15) & ~15ull;
-    const unsigned long long end = total & ~15ull;
-    if (b > end) b = end;
-    if (b > a)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"((const char *)base + a), "r"((unsigned)(b - a))
-                     : "memory");
 }
 
 // NARROW: f < 2^62 and the best f < 2^64 when the cluster starts, so every
@@ -466,6 +376,12 @@ __device__ __forceinline__ void cluster_body(const PeelArgs &A, const int P, uns
         pre = pre && fast;
     }
     int err = werr;
+    // Once the live set fits the dense tail and a minimum-rule round has
+    // closed, the dense tail takes over (its rounds take a fraction of the time
+    // whatever the arcs): the survivors' weights go back to memory, and the
+    // survivors are listed for its build.  A collapsing live set goes back to
+    // the grid-wide rounds the same way.
+    int hand = ST_DONE;
     while (!R.done && !err) {
         if (R.i > A.max_rounds) {
             err = DUPIN_ERR_NO_PROGRESS;
@@ -802,15 +718,37 @@ __device__ __forceinline__ void cluster_body(const PeelArgs &A, const int P, uns
             err = DUPIN_ERR_NO_PROGRESS;
             break;
         }
+        const bool was_min = R.minrule != 0;
         R = tail_plan<NARROW>(A.kD, A.D, A.use_min, A.gpo, A.lpo, st, Mn);
         fast = R.minrule && !over;
         pre = pre && fast;
+        if (was_min && R.minrule && st.size <= A.dcap) {
+            hand = ST_DENSE;
+            break;
+        }
+        if (A.again && !was_min && !R.minrule && !R.done && Un >= DUPIN_AGAIN_ROUND) {
+            hand = ST_RUNNING;
+            break;
+        }
     }
     if (tid == 0 && S.err) set_error(ctl, S.err);
+    int *nlive = ctl->live_sel ? A.live0 : A.live1;
     // peel rounds of this CTA's vertices
-    for (long long s = tid; s < nown; s += CL_THREADS) {
-        const long long wv = tw[s];
-        if (wv < 0) A.pr[live[s * C + r]] = (int)(-wv);
+    for (long long s0 = wid * 32; s0 < nown; s0 += CL_THREADS) {
+        const long long s = s0 + lane;
+        const long long wv = s < nown ? tw[s] : -1;
+        const int u = s < nown ? live[s * C + r] : 0;
+        if (s < nown && wv < 0) A.pr[u] = (int)(-wv);
+        if (hand != ST_DONE) {
+            const unsigned bal = __ballot_sync(0xffffffffu, wv >= 0);
+            int base = 0;
+            if (lane == 0 && bal) base = atomicAdd(&ctl->live_next, __popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (wv >= 0) {
+                nlive[base + __popc(bal & ((1u << lane) - 1u))] = u;
+                A.w[u] = wv;
+            }
+        }
     }
     if (r == 0 && tid == 0) {
         if (err) set_error(ctl, err);
@@ -829,7 +767,17 @@ __device__ __forceinline__ void cluster_body(const PeelArgs &A, const int P, uns
         ctl->tail_ctas = (int)C;
     }
     cl_sync();  // no CTA leaves while another may still read its shared memory
-    if (r == 0 && tid == 0 && !err) ctl->status = ST_DONE;
+    if (r == 0 && tid == 0 && !err) {
+        if (hand != ST_DONE) {
+            ctl->live_len = st.size;
+            ctl->live_sel ^= 1;
+            ctl->live_next = 0;
+            ctl->handed = 1;
+            ctl->bar_count = 0;
+            ctl->minw = R.minw;
+        }
+        ctl->status = hand;
+    }
 }
 
 __global__ void __launch_bounds__(CL_THREADS, 1) k_peel_cluster(PeelArgs A, int P) {

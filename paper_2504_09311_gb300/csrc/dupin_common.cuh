@@ -34,13 +34,22 @@ typedef unsigned __int128 u128;
 #define DUPIN_ONE_CTA_ARCS (1LL << 20)
 // ... provided its live sub-graph fits the tail's arc buffer (2^27 arcs)
 #define DUPIN_TAIL_BUF_ARCS (1LL << 27)
+// On graphs of at least this many arcs the cluster tail gives the peel back to
+// the grid-wide rounds when the live set collapses: a threshold round of this
+// many vertices, with another threshold round to follow.  (R-MAT scale 24, FD:
+// after 2,900 small rounds at 54,000 vertices, ten rounds take 41,000; the
+// cluster's 16 SMs need 9.0 ms for them, the grid-wide rounds 0.6 ms.  The
+// launches that allow it cost about 25 us.)
+#define DUPIN_AGAIN_ARCS (1LL << 27)
+#define DUPIN_AGAIN_ROUND 256
 #define DUPIN_GRP_STRIDE 17  // per tail row: its first arc, then each owner group's end (16 owners at most)
 
 // Peeling phases recorded in PeelCtl::status
 #define ST_RUNNING 0
 #define ST_DONE 1
 #define ST_TAIL 2     // the one-CTA tail finishes the peel
-#define ST_CLUSTER 3  // the cluster tail finishes the peel
+#define ST_CLUSTER 3  // the cluster tail finishes the peel, or hands over to the dense tail
+#define ST_DENSE 4    // the dense tail finishes the peel
 
 // Device-resident control block of one peel.  'bar_*' is the grid barrier;
 // the rest is the state after the last completed round.
@@ -72,8 +81,11 @@ struct PeelCtl {
     // loading checks (the initial-weight pass with its checks on): a row not
     // strictly increasing, and the symmetry fingerprint (0 when symmetric)
     int check_unsorted;
-    int beside_cluster;  // a batched call's earlier peel is on a cluster tail: the grid-wide rounds run narrow
+    int pad1;
     unsigned long long check_fp;
+    unsigned long long check_or;  // all arc weights, or-ed
+    int live_next;      // survivors listed by a cluster tail that hands the peel on ...
+    int handed;         // ... and whether one did
 };
 
 // Per-block partial results of one bulk round (one 128-byte line each)
@@ -155,7 +167,30 @@ struct PeelArgs {
     // G = DUPIN_GRP_STRIDE
     unsigned *tgrp;
     int cl_c;           // CTAs of the cluster tail (0: none)
+    // dense tail: its matrix (in the sparse tail's arc buffer), bytes per
+    // element (1, 4 or 8), the low zero bits left out of an element, and the
+    // most live vertices whose matrix fits there (0: no dense tail)
+    void *dmat;
+    int desz, dshift;
+    int again;          // the cluster tail may give a collapsing graph back to the grid-wide rounds
+    long long dcap;
 };
+
+// The dense tail: CTA r of C owns the columns [r S, (r + 1) S) of a row of C S
+// elements, at most 16 columns per thread.
+#define DN_THREADS 128
+#define DN_MAX_SLICE (16 * DN_THREADS)
+
+// S for L live vertices over C CTAs (a multiple of 16)
+__host__ __device__ __forceinline__ long long dense_slice(long long L, int C) {
+    return ((L + C - 1) / C + 15) & ~15LL;
+}
+
+// the tail that takes 'size' live vertices with 'arcs' live arcs
+__host__ __device__ __forceinline__ int tail_status(const PeelArgs &A, long long size, long long arcs) {
+    if (size <= A.tail_cap && arcs <= A.one_arcs) return ST_TAIL;
+    return size <= A.dcap ? ST_DENSE : ST_CLUSTER;
+}
 
 // ---------------------------------------------------------------- helpers
 

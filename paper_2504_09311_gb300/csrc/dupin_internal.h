@@ -47,6 +47,8 @@ struct PeelWorkspace {
     unsigned *tgrp = nullptr;
     int *tcol = nullptr;
     long long *tcw = nullptr;
+    uint8_t *tbuf = nullptr;  // holds tcw and tcol, or the dense tail's matrix
+    long long tbuf_bytes = 0;
     uint8_t *mask = nullptr;
     bool async = false;  // allocated with cudaMallocAsync (freed with cudaFreeAsync)
     // DUPIN_TIMING: init start, init done, grid-wide rounds start and done,
@@ -64,6 +66,7 @@ struct dupin_graph {
     long long *a = nullptr;
     int *hubs = nullptr;  // hub number -> vertex id (arcs to hubs are stored as -(h + 1))
     int n_hubs = 0;
+    unsigned long long w_or = 0;  // all arc weights, or-ed (0 without weights)
     long long bytes = 0;
     PeelWorkspace *ws = nullptr;
     std::vector<PeelWorkspace *> ws_more;  // further workspaces for concurrent peels of this graph
@@ -99,7 +102,11 @@ int enqueue_peel(const dupin_graph *g, PeelWorkspace *ws, const dupin_params *p,
 // The stages of one peel: PEEL_INIT = control reset and initial weights,
 // PEEL_BULK = the grid-wide rounds (a cooperative launch over the whole GPU),
 // PEEL_BUILD = the tail sub-graph, PEEL_TAIL = the one-CTA rounds.
-enum { PEEL_INIT = 1, PEEL_BUILD = 2, PEEL_TAIL = 4, PEEL_BULK = 8, PEEL_FRONT = 9, PEEL_ALL = 15 };
+// PEEL_BULK2 and PEEL_TAIL2 = the same again, for a peel that the cluster tail
+// gave back (nothing to do otherwise, see peel_again).
+enum { PEEL_INIT = 1, PEEL_BUILD = 2, PEEL_TAIL = 4, PEEL_BULK = 8, PEEL_FRONT = 9, PEEL_BULK2 = 16, PEEL_TAIL2 = 32,
+       PEEL_ALL = 63 };
+bool peel_again(const dupin_graph *g, const dupin_params *p, const PeelPlan &plan);
 // 'init_from' (stage PEEL_INIT only): a workspace whose initial weights for
 // the same graph and metric are already computed on this stream and not yet
 // changed by its grid-wide rounds; they are copied instead of recomputed.
@@ -132,10 +139,14 @@ int launch_small_graph_peel(const PeelArgs &A, int metric, bool check, cudaStrea
 // its CTAs per cluster, and its launch (the kernel returns at once unless the
 // peel's status says the cluster finishes it)
 long long cluster_cap_limit();
-// records in 'next' whether 'prev' (its grid-wide rounds enqueued on s) went to the cluster tail
-void enqueue_note_cluster(const PeelWorkspace *prev, PeelWorkspace *next, cudaStream_t s);
 int cluster_ctas();
 int launch_cluster_tail(const PeelArgs &A, cudaStream_t s);
+// the dense tail (dense.cu): its matrix from the live rows, and its rounds
+// (both return at once unless the peel's status says so)
+// the most live vertices whose matrix fits 'bytes' (esz bytes per element, C CTAs)
+long long dense_cap(long long bytes, int esz, int C);
+int launch_dense_build(const PeelArgs &A, int sms, cudaStream_t s);
+int launch_dense_tail(const PeelArgs &A, cudaStream_t s);
 
 // dupin_peel under the clique metrics TDS and kCLiDS (tds.cu)
 int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_t s);

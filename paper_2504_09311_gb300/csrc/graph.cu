@@ -389,6 +389,7 @@ extern "C" int dupin_graph_load(const dupin_graph_desc *d, void *stream, dupin_g
                                   : "invalid graph: the CSR is not symmetric (an arc without a reverse arc of "
                                     "equal weight)");
         }
+        if (has_w) g->w_or = hc.check_or;
     }
 #undef TRY
     gfree(bad, s);

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
     // chunks through the last arc seen, across warps through the arc before
     // the range) and the symmetry fingerprint
     bool unsorted = false;
-    unsigned long long fp = 0;
+    unsigned long long fp = 0, wor = 0;
     long long prev_row = -1;
     int prev_col = 0;
     if (CHECK && g.rp[r] < we0) {  // the range starts inside row r: compare with the arc before it
@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         const bool valid = x < we1;
         if (CHECK && valid) {
             if (cvx < 0 || cvx >= n || val < 0) bad = true;
+            wor |= (unsigned long long)val;
         }
         // fast path: the whole chunk lies in row r (long rows, hubs)
         const long long cend = x0 + 32 < we1 ? x0 + 32 : we1;
@@ -263,6 +264,9 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         if (__any_sync(0xffffffffu, unsorted) && lane == 0) atomicExch(&ctl->check_unsorted, 1);
         for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);  // wrapping sum
         if (lane == 0 && fp) atomicAdd(&ctl->check_fp, fp);
+        const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)wor);
+        const unsigned oh = __reduce_or_sync(0xffffffffu, (unsigned)(wor >> 32));
+        if (lane == 0) atomicOr(&ctl->check_or, ((unsigned long long)oh << 32) | ol);
     }
 }
 
@@ -338,7 +342,7 @@ __global__ void k_init_finish(PeelArgs A, long long n) {
     c->tail_ctas = 0;
     if (n == 0) c->status = ST_DONE;
     else if (n <= A.hcap && A.g.arcs <= A.tail_arcs)
-        c->status = n <= A.tail_cap && A.g.arcs <= A.one_arcs ? ST_TAIL : ST_CLUSTER;
+        c->status = tail_status(A, n, A.g.arcs);
     else c->status = ST_RUNNING;
     if (A.tr_cap > 0) {
         A.tr_f_hi[0] = (long long)c->f_hi;
@@ -907,42 +911,28 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         ctl->gpo_lt = st.gpo_lt;
         ctl->n_min_rule = st.n_min_rule;
         ctl->scan_volume = st.scan;
-        ctl->bulk_rounds = st.round;
+        if (!ctl->handed) ctl->bulk_rounds = st.round;
         ctl->elive = s_elive;
         if (ctl->error == 0)
-            ctl->status = st.size == 0 ? ST_DONE
-                          : (st.size <= A.tail_cap && 2 * s_elive <= A.one_arcs ? ST_TAIL : ST_CLUSTER);
+            ctl->status = st.size == 0 ? ST_DONE : tail_status(A, st.size, 2 * s_elive);
     }
 }
 
-// Beside a cluster tail (a batched call's earlier peel) the rounds run on a
-// quarter of the launched blocks and the rest leave at once: the cluster's
-// rounds are bound by the latency of their loads, which a full-width stage's
-// memory traffic raises.  The flag is set before the launch, so every block
-// reads the same value.
 __global__ void __launch_bounds__(BULK_THREADS, 1) k_peel_bulk(PeelArgs A) {
-    unsigned G = gridDim.x;
-    if (A.ctl->beside_cluster) G = G / 4 > 0 ? G / 4 : 1;
-    if (blockIdx.x >= G) return;
-    peel_bulk_body(A, blockIdx.x, G);
-}
-
-// a later peel of a batched call learns whether this one's tail is a cluster
-// (read right after this peel's grid-wide rounds, before its tail starts)
-__global__ void k_note_cluster(const PeelCtl *prev, PeelCtl *next) {
-    if (prev->status == ST_CLUSTER) next->beside_cluster = 1;
-}
-
-void enqueue_note_cluster(const PeelWorkspace *prev, PeelWorkspace *next, cudaStream_t s) {
-    k_note_cluster<<<1, 1, 0, s>>>(prev->ctl, next->ctl);
+    peel_bulk_body(A, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------- (d) tail sub-graph
 
+// does the build of the sparse tails (dense 0) or of the dense tail (1) run?
+__device__ __forceinline__ bool builds(const PeelCtl *c, int dense) {
+    return (dense ? c->status == ST_DENSE : c->status == ST_TAIL || c->status == ST_CLUSTER) && !c->error;
+}
+
 // local ids and full degrees of the live vertices
-__global__ void k_tail_prep(PeelArgs A) {
+__global__ void k_tail_prep(PeelArgs A, int dense) {
     const PeelCtl *c = A.ctl;
-    if ((c->status != ST_TAIL && c->status != ST_CLUSTER) || c->error) return;
+    if (!builds(c, dense)) return;
     const long long L = c->live_len;
     const int *live = c->live_sel ? A.live1 : A.live0;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < L; p += (long long)gridDim.x * blockDim.x) {
@@ -953,10 +943,10 @@ __global__ void k_tail_prep(PeelArgs A) {
 }
 
 // exclusive prefix of x[0..L) in place, x[L] = total (one block)
-__global__ void __launch_bounds__(SCAN_THREADS) k_tail_scan(PeelArgs A, long long *x, const int *cnt) {
+__global__ void __launch_bounds__(SCAN_THREADS) k_tail_scan(PeelArgs A, long long *x, const int *cnt, int dense) {
     __shared__ long long s_w[SCAN_THREADS / 32];
     const PeelCtl *c = A.ctl;
-    if ((c->status != ST_TAIL && c->status != ST_CLUSTER) || c->error) return;
+    if (!builds(c, dense)) return;
     const long long L = c->live_len;
     long long carry = 0;
     for (long long b0 = 0; b0 < L; b0 += SCAN_THREADS) {
@@ -970,7 +960,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tail_scan(PeelArgs A, long lon
     if (threadIdx.x == 0) {
         x[L] = carry;
         if (cnt) {
-            A.ctl->tail_arcs = carry;
+            if (!c->handed) A.ctl->tail_arcs = carry;
             if (carry > A.tarc_cap) set_error(A.ctl, DUPIN_ERR_OOM);
         }
     }
@@ -983,7 +973,7 @@ __global__ void __launch_bounds__(BULK_THREADS) k_tail_arcs(PeelArgs A) {
     __shared__ long long s_start[WALK_WIN + 1];
     __shared__ long long s_k0;
     const PeelCtl *c = A.ctl;
-    if ((c->status != ST_TAIL && c->status != ST_CLUSTER) || c->error) return;
+    if (!builds(c, 0)) return;
     const long long L = c->live_len;
     const int *live = c->live_sel ? A.live1 : A.live0;
     const long long tot = A.tdeg[L];
@@ -1503,7 +1493,7 @@ void workspace_free(PeelWorkspace *ws, cudaStream_t s) {
     void *ptrs[] = {ws->w, ws->pr, ws->live0, ws->live1, ws->stage_id, ws->stage_start, ws->stage_off,
                     ws->fstart, ws->fbase, ws->cstart, ws->part, ws->ctl, ws->tr_f_hi, ws->tr_f_lo,
                     ws->tr_size, ws->tr_peeled, ws->loc, ws->tdeg, ws->tlrp, ws->tcnt, ws->tfill,
-                    ws->tgrp, ws->tcol, ws->tcw, ws->mask};
+                    ws->tgrp, ws->tbuf, ws->mask};
     for (void *q : ptrs) {
         if (!q) continue;
         if (ws->async) cudaFreeAsync(q, s);
@@ -1557,8 +1547,12 @@ PeelWorkspace *workspace_create(long long n, long long arcs, bool has_cw, const 
     A(&ws->tcnt, tail_cap + 1);
     A(&ws->tfill, tail_cap + 1);
     A(&ws->tgrp, (tail_cap + 1) * DUPIN_GRP_STRIDE);
-    A(&ws->tcol, ws->tarc_cap);
-    if (has_cw) A(&ws->tcw, ws->tarc_cap);
+    // the tail's arcs: weights, then heads (one block: the dense tail's matrix takes their place)
+    const long long wbytes = has_cw ? (8 * ws->tarc_cap + 255) & ~255LL : 0;
+    ws->tbuf_bytes = (wbytes + 4 * ws->tarc_cap) & ~15LL;
+    A(&ws->tbuf, wbytes + 4 * ws->tarc_cap);
+    if (has_cw) ws->tcw = (long long *)ws->tbuf;
+    ws->tcol = (int *)(ws->tbuf + wbytes);
     A(&ws->mask, n);
     if (e != cudaSuccess) {
         workspace_free(ws, s);
@@ -1700,7 +1694,25 @@ static PeelArgs make_args(const dupin_graph *g, const PeelWorkspace *ws, const d
     A.tarc_cap = ws->tarc_cap;
     A.tgrp = ws->tgrp;
     A.cl_c = plan.cl_cap > 0 ? cluster_ctas() : 0;
+    A.dmat = ws->tbuf;
+    A.again = 0;
+    {  // the dense tail's element: the weights without their common low zero bits
+        const unsigned long long o = p->metric == DUPIN_DG ? (unsigned long long)DUPIN_Q_ONE : g->w_or;
+        A.dshift = o ? __builtin_ctzll(o) : 0;
+        A.desz = (o >> A.dshift) >> 32 ? 8 : ((o >> A.dshift) >> 8 ? 4 : 1);
+        if (A.desz == 8) A.dshift = 0;
+    }
+    // (without the minimum rule a peel has few rounds, and the dense tail's
+    // launches would cost more than it gains)
+    A.dcap = plan.cl_cap > 0 && A.use_min && g->arcs > DUPIN_ONE_CTA_ARCS
+                 ? dense_cap(ws->tbuf_bytes, A.desz, A.cl_c) : 0;
     return A;
+}
+
+// may the cluster tail give this peel back to the grid-wide rounds?
+bool peel_again(const dupin_graph *g, const dupin_params *p, const PeelPlan &plan) {
+    const bool use_min = (long long)p->k_mult * (p->eps_den + p->eps_num) < 2 * p->eps_den;
+    return plan.cl_cap > 0 && use_min && g->arcs >= DUPIN_AGAIN_ARCS;
 }
 
 // Enqueue a whole peel on 'stream' (no host synchronisation).
@@ -1754,49 +1766,72 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
         k_init_finish<<<1, 1, 0, s>>>(A, g->n);
         if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[1], s));
     }
-    if (stages & PEEL_BULK) {
-        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[2], s));
-        if (g->n > A.hcap || g->arcs > A.tail_arcs) {
-            const int grid = bulk_grid > 0 && bulk_grid < ws->grid ? bulk_grid : ws->grid;
-            void *args[] = {&A};
-            cudaError_t e =
-                cudaLaunchCooperativeKernel((void *)k_peel_bulk, dim3(grid), dim3(BULK_THREADS), args, 0, s);
-            if (e != cudaSuccess) return dupin_cuda_fail(e, "cooperative launch of k_peel_bulk");
-        }
-        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[3], s));
-    }
-    if (stages & PEEL_BUILD) {
-        int sms = 0, dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[4], s));
+    const bool again = peel_again(g, p, plan);
+    auto bulk = [&]() -> int {
+        const int grid = bulk_grid > 0 && bulk_grid < ws->grid ? bulk_grid : ws->grid;
+        void *args[] = {&A};
+        cudaError_t e = cudaLaunchCooperativeKernel((void *)k_peel_bulk, dim3(grid), dim3(BULK_THREADS), args, 0, s);
+        return e == cudaSuccess ? DUPIN_OK : dupin_cuda_fail(e, "cooperative launch of k_peel_bulk");
+    };
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // the sparse tails' sub-graph
+    auto build = [&]() -> int {
         DUPIN_CUDA_TRY(cudaMemsetAsync(ws->tcnt, 0, sizeof(int) * (size_t)(tail_cap + 1), s));
         DUPIN_CUDA_TRY(cudaMemsetAsync(ws->tfill, 0, sizeof(int) * (size_t)(tail_cap + 1), s));
         if (A.cl_c > 0)
             DUPIN_CUDA_TRY(cudaMemsetAsync(ws->tgrp, 0, sizeof(unsigned) * (size_t)(tail_cap + 1) * DUPIN_GRP_STRIDE, s));
-        k_tail_prep<<<sms * 2, 256, 0, s>>>(A);
-        k_tail_scan<<<1, SCAN_THREADS, 0, s>>>(A, ws->tdeg, nullptr);
+        k_tail_prep<<<sms * 2, 256, 0, s>>>(A, 0);
+        k_tail_scan<<<1, SCAN_THREADS, 0, s>>>(A, ws->tdeg, nullptr, 0);
         k_tail_arcs<0><<<sms * 2, BULK_THREADS, 0, s>>>(A);
         if (A.cl_c > 0) k_tail_rowcnt<<<sms, 256, 0, s>>>(A);
         // tcnt -> tlrp
-        PeelArgs A2 = A;
-        k_tail_scan<<<1, SCAN_THREADS, 0, s>>>(A2, ws->tlrp, ws->tcnt);
+        k_tail_scan<<<1, SCAN_THREADS, 0, s>>>(A, ws->tlrp, ws->tcnt, 0);
         if (A.cl_c > 0) k_tail_grp<<<sms, 256, 0, s>>>(A);
         k_tail_arcs<1><<<sms * 2, BULK_THREADS, 0, s>>>(A);
+        return DUPIN_OK;
+    };
+    // the status the stage before left picks one of the tails; the others
+    // return at once
+    auto tails = [&]() -> int {
+        int rc2;
+        if (plan.tail_cap > 0) {
+            if ((rc2 = set_tail_smem())) return rc2;
+            k_peel_tail<<<1, TAIL_THREADS, (size_t)tail_smem_bytes(plan.tail_cap), s>>>(A);
+        }
+        if (plan.cl_cap > 0 && (rc2 = launch_cluster_tail(A, s))) return rc2;
+        if (A.dcap > 0) {  // from the grid-wide rounds, or after the cluster tail
+            k_tail_prep<<<sms * 2, 256, 0, s>>>(A, 1);
+            k_tail_scan<<<1, SCAN_THREADS, 0, s>>>(A, ws->tdeg, nullptr, 1);
+            if ((rc2 = launch_dense_build(A, sms, s))) return rc2;
+            if ((rc2 = launch_dense_tail(A, s))) return rc2;
+        }
+        return DUPIN_OK;
+    };
+    if (stages & PEEL_BULK) {
+        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[2], s));
+        if (g->n > A.hcap || g->arcs > A.tail_arcs) {
+            if ((rc = bulk())) return rc;
+        }
+        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[3], s));
+    }
+    if (stages & PEEL_BUILD) {
+        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[4], s));
+        if ((rc = build())) return rc;
         if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[5], s));
     }
     if (stages & PEEL_TAIL) {
-        // the status the grid-wide stage (or the set-up) left picks one of
-        // the two tails; the other returns at once
-        if (plan.tail_cap > 0) {
-            rc = set_tail_smem();
-            if (rc) return rc;
-            k_peel_tail<<<1, TAIL_THREADS, (size_t)tail_smem_bytes(plan.tail_cap), s>>>(A);
-        }
-        if (plan.cl_cap > 0) {
-            rc = launch_cluster_tail(A, s);
-            if (rc) return rc;
-        }
+        A.again = again ? 1 : 0;
+        if ((rc = tails())) return rc;
+        A.again = 0;
+        if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[6], s));
+    }
+    if (again && (stages & PEEL_BULK2)) {
+        if ((rc = bulk())) return rc;
+    }
+    if (again && (stages & PEEL_TAIL2)) {
+        if ((rc = build()) || (rc = tails())) return rc;
         if (timing) DUPIN_CUDA_TRY(cudaEventRecord(ws->ev[6], s));
     }
     cudaError_t e = cudaGetLastError();
