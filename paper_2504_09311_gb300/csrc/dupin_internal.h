@@ -91,6 +91,9 @@ void workspace_free(PeelWorkspace *ws, cudaStream_t s);
 void workspace_release(PeelWorkspace *ws);
 // release the freed graph buffers the library's memory pool keeps (current device)
 void graph_pool_trim();
+// stream-ordered device memory from that pool
+cudaError_t graph_pool_alloc(void **p, size_t bytes, cudaStream_t s);
+void graph_pool_free(void *p, cudaStream_t s);
 int workspace_ensure(dupin_graph *g, const PeelPlan &plan);
 // workspace k of graph g (0: the one dupin_peel uses), allocated or grown for plan
 PeelWorkspace *workspace_slot(dupin_graph *g, int k, const PeelPlan &plan, int *rc);

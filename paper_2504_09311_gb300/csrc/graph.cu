@@ -64,6 +64,9 @@ static void gfree(void *p, cudaStream_t s) {
     if (p) cudaFreeAsync(p, s);
 }
 
+cudaError_t graph_pool_alloc(void **p, size_t bytes, cudaStream_t s) { return galloc(p, bytes, s); }
+void graph_pool_free(void *p, cudaStream_t s) { gfree(p, s); }
+
 void graph_pool_trim() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;

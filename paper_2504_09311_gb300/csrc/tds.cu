@@ -6,49 +6,75 @@
 // Algorithm 4's trims by flag, exactly as for the other metrics but on plain
 // counts (no Q32.32 scale): every comparison is between ratios of integers.
 //
-// Device state lives in one control block; a round is five launches --
-//   min     the minimum live weight (the minimum rule and the trim test);
-//   plan    one thread: a trim round if some live w < g(S) (Algorithm 4),
-//           else a main round (w <= max(tau_max, k(1+eps) g)), or the
-//           minimum rule if that threshold selects nobody;
+// Device state lives in one control block; a round is four launches --
 //   select  every live u with w_u <= T leaves: its round is recorded and it
 //           joins the round's list;
-//   expand  one warp per removed vertex u, one lane per arc u -> v with v in
-//           S_{i-1}: the cliques of G[S_{i-1}] through u whose smallest
-//           member besides u is v (for TDS a merge of the two sorted rows,
-//           the common neighbours x > v, each triangle counted by its
-//           smallest member in U_i; for kCLiDS a depth-first walk over u's
-//           row after v, each candidate kept when it is in the rows of every
-//           member chosen so far and, if it leaves in this round too,
-//           outranks u in (degree, id), so that only the removed member of
-//           lowest rank lists the clique); each clique that dies lowers f by
-//           one and each member outside U_i by one;
-//   close   one thread: f, |S|, the trace, the best prefix.
-// The host launches rounds in groups and reads the control block between
-// groups; launches after the peel ends return at once.  The initial counts
-// list every clique once: TDS from its smallest vertex, kCLiDS from its
-// member of lowest degree (the same walks, keeping only members that outrank
-// u).  Rows are sorted (the loader checks it).
+//   expand  the cliques of G[S_{i-1}] that die, listed once each (below), in
+//           two launches by the size of a vertex's candidate set; each lowers
+//           f by one and each member outside U_i by one;
+//   close   the minimum live weight; the last block closes the round (f, |S|,
+//           the trace, the best prefix) and plans the next one: a trim round
+//           if some live w < g(S) (Algorithm 4), else a main round (w <=
+//           max(tau_max, k(1+eps) g)), or the minimum rule if that threshold
+//           selects nobody.
+// The host launches rounds in groups (2, 4, 8, ... 32) and reads the control
+// block between groups; launches after the peel ends return at once.
+//
+// Listing.  A clique belongs to its member u of lowest rank = (degree, id); a
+// dying one to its removed member of lowest rank.  u's candidates P are its
+// neighbours that may be the others: those that outrank u, or in a round the
+// ones in S_{i-1} that survive it or outrank u.  The cliques of u are the
+// (q-1)-cliques of G[P], and the ones through v in P are the (q-2)-cliques of
+// G[P] among v's neighbours: popcounts over ANDed rows of P's adjacency
+// matrix in shared memory, so no clique is visited one by one and w is
+// updated once per (u, v).  Whether two candidates are adjacent comes from one
+// bit of a global matrix over the (at most) CORE_MAX vertices of highest
+// degree, or from a binary search in the row of the one outside it, a short
+// row.  (A row merge or a leapfrog walk per arc, one warp per u, read hub
+// rows of thousands for every arc of a hub.  One peel, k = q: R-MAT scale 15
+// TDS 63.4 -> 1.57 ms, scale 13 4-cliques 417 -> 0.90 ms; what is left is bound
+// by the latency of the bit lookups and row searches, 64 warps per SM.)
+// A warp takes a vertex of at most WARP_P candidates, a CTA one of up to
+// CTA_P (one SM's shared memory; for triangles, which need no matrix, P
+// itself is the limit); larger ones fall back to a depth-first walk over the
+// rows.  Rows are sorted (the loader checks it).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 
 #include "dupin_internal.h"
 
 namespace {
 
+constexpr int QMAX = DUPIN_CLIQUE_MAX_Q;
+constexpr int CORE_MAX = 8192;             // vertices of the adjacency matrix (8 MB)
+constexpr int CORE_WORDS = CORE_MAX / 32;  // its row
+constexpr int DEG_BINS = 4096;
+constexpr int WARP_P = 128;                // candidates of a warp's vertex
+constexpr int WARP_STRIDE = WARP_P / 32 + 1;
+constexpr int CTA_P = 1216;                // candidates of a CTA's vertex with a matrix ...
+constexpr int CTA_P3 = 24576;              // ... and without (triangles)
+constexpr int WARP_TEAM = 256, CTA_TEAM = 512;
+constexpr size_t CTA_SMEM = 2 * 4 * CTA_P + 4 * (size_t)CTA_P * (CTA_P / 32 + 1);
+static_assert((CTA_P / 32 + 1) % 2 == 1 && WARP_STRIDE % 2 == 1, "an odd row stride spreads rows over the banks");
+static_assert(2 * 4 * (size_t)CTA_P3 <= CTA_SMEM, "triangles' candidates fit the same shared memory");
+
 struct TdsCtl {
     long long round, size, best_round, best_size, n_min_rule;
-    long long f, bf;           // triangle counts
+    long long f, bf;           // clique counts
     long long gpo_le, gpo_lt;  // tau_max's integer forms (Algorithm 3)
     long long T;               // this round removes live w <= T
     long long kind;            // 0 main round, 1 minimum rule, 2 trim round
     long long minw;            // minimum live weight before the round
     long long ucnt;            // |U_i|
-    long long df;              // triangles that die in the round
+    long long df;              // cliques that die in the round
     int status;                // 0 running, 1 done
     int error;
+    int nbig;                  // vertices left to the CTA launch
+    int blocks;                // blocks of the closing launch that are through
+    int core_thr, ncore;       // the adjacency matrix takes degrees >= core_thr
 };
 
 struct TdsArgs {
@@ -59,6 +85,10 @@ struct TdsArgs {
     long long *w;
     int *pr;
     int *front;
+    int *big;        // vertices left to the CTA launch
+    int *ci;         // row of the adjacency matrix, -1: none
+    unsigned *bits;  // [CORE_MAX][CORE_WORDS]
+    int *hist;       // [DEG_BINS]
     TdsCtl *ctl;
     long long *tr_f, *tr_size, *tr_peeled;
     long long tr_cap;
@@ -81,49 +111,93 @@ __device__ __forceinline__ long long row_after(const TdsArgs &A, int v, int x) {
     return lo;
 }
 
+__device__ __forceinline__ bool in_row(const TdsArgs &A, int v, int x) {
+    const long long p = row_after(A, v, x - 1);
+    return p < A.rp[v + 1] && head(A, p) == x;
+}
+
+// are x and y adjacent?  cx, cy: their rows of the adjacency matrix, or -1
+__device__ __forceinline__ bool adjacent(const TdsArgs &A, int x, int cx, int y, int cy) {
+    if (cx >= 0 && cy >= 0) return (A.bits[cx * CORE_WORDS + (cy >> 5)] >> (cy & 31)) & 1u;
+    return cx < 0 ? in_row(A, x, y) : in_row(A, y, x);
+}
+
+// ------------------------------------------------------------------ set-up
+
 __global__ void k_tds_reset(TdsArgs A) {
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < A.n; u += (long long)gridDim.x * blockDim.x) {
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, dt = (long long)gridDim.x * blockDim.x;
+    for (long long u = t0; u < A.n; u += dt) {
         A.w[u] = 0;
         A.pr[u] = DUPIN_LIVE;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    for (long long x = t0; x < DEG_BINS; x += dt) A.hist[x] = 0;
+    if (t0 == 0) {
         TdsCtl z;
         memset(&z, 0, sizeof(z));
         z.gpo_lt = -1;
         z.size = A.n;
+        z.minw = 0x7fffffffffffffffLL;
         *A.ctl = z;
     }
 }
 
-// every triangle u < v < x once (one warp per u, one lane per arc u -> v, v > u)
-__global__ void k_tds_count(TdsArgs A) {
+__global__ void k_core_hist(TdsArgs A) {
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < A.n; u += (long long)gridDim.x * blockDim.x) {
+        const long long d = A.rp[u + 1] - A.rp[u];
+        atomicAdd(&A.hist[d < DEG_BINS - 1 ? (int)d : DEG_BINS - 1], 1);
+    }
+}
+
+// the lowest degree at which no more than CORE_MAX vertices lie (one block of
+// 1024: four bins per thread, a scan from the top)
+__global__ void __launch_bounds__(1024) k_core_threshold(TdsArgs A) {
+    __shared__ long long s_w[32];
+    __shared__ int s_best;
+    const int t = threadIdx.x;
+    if (t == 0) s_best = 0x7fffffff;
+    const int b0 = DEG_BINS - 4 * (t + 1);  // this thread's bins b0 .. b0 + 3
+    long long c[4], sum = 0;
+    for (int k = 3; k >= 0; k--) {
+        c[k] = A.hist[b0 + k];
+        sum += c[k];
+    }
+    long long incl = warp_incl_scan64(sum);
+    if ((t & 31) == 31) s_w[t >> 5] = incl;
+    __syncthreads();
+    long long above = incl - sum;
+    for (int k = 0; k < (t >> 5); k++) above += s_w[k];
+    for (int k = 3; k >= 0; k--) {
+        above += c[k];
+        if (above > CORE_MAX) break;
+        atomicMin(&s_best, b0 + k);
+    }
+    __syncthreads();
+    if (t == 0) A.ctl->core_thr = s_best;
+}
+
+__global__ void k_core_rows(TdsArgs A) {
+    const int thr = A.ctl->core_thr;
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < A.n; u += (long long)gridDim.x * blockDim.x) {
+        const long long d = A.rp[u + 1] - A.rp[u];
+        A.ci[u] = d >= thr ? atomicAdd(&A.ctl->ncore, 1) : -1;
+    }
+}
+
+// a warp per core vertex clears its row and sets its neighbours' bits
+__global__ void k_core_bits(TdsArgs A) {
     const int lane = threadIdx.x & 31;
     const long long W = (long long)gridDim.x * (blockDim.x >> 5);
-    long long cnt = 0;
     for (long long u = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); u < A.n; u += W) {
-        const long long b = A.rp[u], e = A.rp[u + 1];
-        for (long long j = b + lane; j < e; j += 32) {
-            const int v = head(A, j);
-            if (v <= (int)u) continue;
-            long long a = j + 1, c = row_after(A, v, v);
-            const long long ce = A.rp[v + 1];
-            while (a < e && c < ce) {
-                const int xa = head(A, a), xc = head(A, c);
-                if (xa < xc) a++;
-                else if (xc < xa) c++;
-                else {
-                    atomicAdd((unsigned long long *)&A.w[u], 1ull);
-                    atomicAdd((unsigned long long *)&A.w[v], 1ull);
-                    atomicAdd((unsigned long long *)&A.w[xa], 1ull);
-                    cnt++;
-                    a++;
-                    c++;
-                }
-            }
+        const int cu = A.ci[u];
+        if (cu < 0) continue;
+        unsigned *row = A.bits + (size_t)cu * CORE_WORDS;
+        for (int k = lane; k < CORE_WORDS; k += 32) row[k] = 0;
+        __syncwarp();
+        for (long long p = A.rp[u] + lane; p < A.rp[u + 1]; p += 32) {
+            const int cv = A.ci[head(A, p)];
+            if (cv >= 0) atomicOr(&row[cv >> 5], 1u << (cv & 31));
         }
     }
-    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    if (lane == 0 && cnt) atomicAdd((unsigned long long *)&A.ctl->f, (unsigned long long)cnt);
 }
 
 __global__ void k_tds_start(TdsArgs A) {
@@ -134,6 +208,7 @@ __global__ void k_tds_start(TdsArgs A) {
     c->best_size = A.n;
     c->bf = c->f;
     c->status = A.n == 0 ? 1 : 0;
+    c->nbig = 0;
     if (A.tr_cap > 0) {
         A.tr_f[0] = c->f;
         A.tr_size[0] = A.n;
@@ -141,127 +216,184 @@ __global__ void k_tds_start(TdsArgs A) {
     }
 }
 
-__global__ void k_tds_min(TdsArgs A) {
-    const TdsCtl *c = A.ctl;
-    if (c->status || c->error) return;
-    long long m = 0x7fffffffffffffffLL;
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < A.n; u += (long long)gridDim.x * blockDim.x)
-        if (A.pr[u] == DUPIN_LIVE && A.w[u] < m) m = A.w[u];
-    m = warp_min64(m);
-    if ((threadIdx.x & 31) == 0 && m != 0x7fffffffffffffffLL) atomicMin(&A.ctl->minw, m);
-}
+// ------------------------------------------------------------------ listing
 
-__device__ __forceinline__ long long tds_floor(u128 x, u128 y) {
-    const u128 q = x / y;
-    return q > (u128)0x7fffffffffffffffULL ? 0x7fffffffffffffffLL : (long long)q;
-}
-
-// ceil(x / y) - 1 (the largest integer strictly below x / y), -1 for x = 0
-__device__ __forceinline__ long long tds_below(u128 x, u128 y) {
-    if (x == 0) return -1;
-    return tds_floor(x - 1, y);
-}
-
-__global__ void k_tds_plan(TdsArgs A) {
-    TdsCtl *c = A.ctl;
-    if (c->status || c->error) return;
-    if (c->round + 1 > A.max_rounds) {
-        c->error = DUPIN_ERR_NO_PROGRESS;
-        return;
+// Which neighbours of u are candidates.  ROUND 0: the initial counts; else the
+// round whose removals are expanded.
+struct Keep {
+    int u, r;  // r < 0: the initial counts
+    long long du;
+    __device__ __forceinline__ Keep(const TdsArgs &A, int u_, int r_) : u(u_), r(r_), du(A.rp[u_ + 1] - A.rp[u_]) {}
+    __device__ __forceinline__ bool outranks(const TdsArgs &A, int x) const {
+        const long long dx = A.rp[x + 1] - A.rp[x];
+        return dx > du || (dx == du && x > u);
     }
-    const u128 f = (u128)(unsigned long long)c->f, size = (u128)(unsigned long long)c->size;
-    const long long m = c->minw;
-    const long long below_g = tds_below(f, size);
-    if (A.lpo && c->round > 0 && m <= below_g) {  // Algorithm 4: some live w < g(S)
-        c->T = below_g > c->gpo_lt ? below_g : c->gpo_lt;
-        c->kind = 2;
-    } else {
-        long long T = tds_floor((u128)(unsigned long long)A.kD * f, (u128)(unsigned long long)A.D * size);
-        if (A.gpo) {  // Algorithm 3: tau_max refined at every main round
-            const u128 num = (u128)(unsigned long long)A.D * f, den = (u128)(unsigned long long)A.kD * size;
-            const long long le = tds_floor(num, den), lt = tds_below(num, den);
-            if (le > c->gpo_le) c->gpo_le = le;
-            if (lt > c->gpo_lt) c->gpo_lt = lt;
-            if (c->gpo_le > T) T = c->gpo_le;
-        }
-        c->kind = 0;
-        if (m > T) {  // the threshold selects nobody: the minimum rule
-            T = m;
-            c->kind = 1;
-        }
-        c->T = T;
+    __device__ __forceinline__ bool operator()(const TdsArgs &A, int x) const {
+        if (r < 0) return outranks(A, x);
+        const int px = A.pr[x];
+        if (px != r) return px > r;  // left in an earlier round, or survives this one
+        return outranks(A, x);
     }
-    c->ucnt = 0;
-    c->df = 0;
+};
+
+// v's share of u's cliques: t of them hold v
+__device__ __forceinline__ void credit(const TdsArgs &A, int v, unsigned long long t, int r) {
+    if (t == 0) return;
+    if (r < 0) atomicAdd((unsigned long long *)&A.w[v], t);
+    else if (A.pr[v] > r) atomicAdd((unsigned long long *)&A.w[v], 0ull - t);
 }
 
-__global__ void k_tds_select(TdsArgs A) {
-    const TdsCtl *c = A.ctl;
-    if (c->status || c->error) return;
-    const long long T = c->T;
-    const int r = (int)(c->round + 1);
-    const int lane = threadIdx.x & 31;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long b = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); b < A.n; b += stride) {
-        const long long u = b + lane;
-        const bool sel = u < A.n && A.pr[u] == DUPIN_LIVE && A.w[u] <= T;
-        const unsigned m = __ballot_sync(0xffffffffu, sel);
-        if (!m) continue;
-        long long base = 0;
-        if (lane == 0) base = (long long)atomicAdd((unsigned long long *)&A.ctl->ucnt, (unsigned long long)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (sel) {
-            A.pr[u] = r;
-            A.front[base + __popc(m & ((1u << lane) - 1u))] = (int)u;
-        }
-    }
-}
-
-__global__ void k_tds_expand(TdsArgs A) {
-    const TdsCtl *c = A.ctl;
-    if (c->status || c->error) return;
-    const int r = (int)(c->round + 1);
-    const long long U = c->ucnt;
-    const int lane = threadIdx.x & 31;
-    const long long W = (long long)gridDim.x * (blockDim.x >> 5);
-    long long dead = 0;
-    for (long long k = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); k < U; k += W) {
-        const int u = A.front[k];
-        const long long b = A.rp[u], e = A.rp[u + 1];
-        for (long long j = b + lane; j < e; j += 32) {
-            const int v = head(A, j);
-            const int pv = A.pr[v];
-            if (pv < r) continue;  // left in an earlier round
-            long long a = j + 1, cc = row_after(A, v, v);
-            const long long ce = A.rp[v + 1];
-            while (a < e && cc < ce) {
-                const int xa = head(A, a), xc = head(A, cc);
-                if (xa < xc) a++;
-                else if (xc < xa) cc++;
-                else {
-                    const int x = xa, px = A.pr[x];
-                    if (px >= r) {  // the triangle {u, v, x} of G[S_{i-1}]
-                        const bool vu = pv == r, xu = px == r;
-                        // counted once: by its smallest member in U_i
-                        if (!((vu && v < u) || (xu && x < u))) {
-                            dead++;
-                            if (!vu) atomicAdd((unsigned long long *)&A.w[v], (unsigned long long)-1ll);
-                            if (!xu) atomicAdd((unsigned long long *)&A.w[x], (unsigned long long)-1ll);
-                        }
-                    }
-                    a++;
-                    cc++;
-                }
+// The M-cliques y_0 < y_1 < ... < y_{M-1} that lie in the rows row[0..D] (D
+// chosen members besides the first row's), from word 'w0' on and above the
+// bits that 'first' leaves in it.
+template <int D, int M>
+__device__ __forceinline__ unsigned long long cliques_in(const unsigned *rows, int stride, int words,
+                                                         const unsigned *(&row)[M], int w0, unsigned first) {
+    unsigned long long t = 0;
+    for (int w = w0; w < words; w++) {
+        unsigned b = row[0][w];
+#pragma unroll
+        for (int k = 1; k <= D; k++) b &= row[k][w];
+        if (w == w0) b &= first;
+        if (D == M - 1) {
+            t += __popc(b);
+        } else {
+            while (b) {
+                const int j = __ffs(b) - 1;
+                b &= b - 1;
+                row[D + 1 < M ? D + 1 : 0] = rows + (size_t)(32 * w + j) * stride;
+                t += cliques_in<(D + 1 < M ? D + 1 : D), M>(rows, stride, words, row, w, j == 31 ? 0u : ~0u << (j + 1));
             }
         }
     }
-    for (int d = 16; d > 0; d >>= 1) dead += __shfl_down_sync(0xffffffffu, dead, d);
-    if (lane == 0 && dead) atomicAdd((unsigned long long *)&A.ctl->df, (unsigned long long)dead);
+    return t;
 }
 
-// ---- kCLiDS: q-cliques, 3 <= q <= DUPIN_CLIQUE_MAX_Q
+// the M-cliques among the neighbours of row 'v' whose first member's word is in
+// [w0, w1) (M >= 2)
+template <int M>
+__device__ __forceinline__ unsigned long long cliques_of(const unsigned *rows, int stride, int words, int v, int w0, int w1) {
+    const unsigned *row[M];
+    row[0] = rows + (size_t)v * stride;
+    unsigned long long t = 0;
+    for (int w = w0; w < w1; w++) {
+        unsigned b = row[0][w];
+        while (b) {
+            const int j = __ffs(b) - 1;
+            b &= b - 1;
+            row[1] = rows + (size_t)(32 * w + j) * stride;
+            t += cliques_in<1, M>(rows, stride, words, row, w, j == 31 ? 0u : ~0u << (j + 1));
+        }
+    }
+    return t;
+}
 
-constexpr int QMAX = DUPIN_CLIQUE_MAX_Q;
+__device__ __forceinline__ unsigned long long cliques_of(int M, const unsigned *rows, int stride, int words, int v, int w0,
+                                                         int w1) {
+    switch (M) {
+        case 2: return cliques_of<2>(rows, stride, words, v, w0, w1);
+        case 3: return cliques_of<3>(rows, stride, words, v, w0, w1);
+        case 4: return cliques_of<4>(rows, stride, words, v, w0, w1);
+        case 5: return cliques_of<5>(rows, stride, words, v, w0, w1);
+        default: return cliques_of<6>(rows, stride, words, v, w0, w1);
+    }
+}
+
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x) {
+    return (unsigned long long)__shfl_sync(0xffffffffu, warp_sum64((long long)x), 0);
+}
+
+// u's cliques by one warp; false when it has more than WARP_P candidates.
+// Adds the sum over v of the cliques through v, (q-1) times u's, to 'sum'.
+__device__ __forceinline__ bool warp_vertex(const TdsArgs &A, int u, int r, int *ids, int *cis, unsigned *rows,
+                                            unsigned long long &sum) {
+    const int lane = threadIdx.x & 31;
+    const Keep keep(A, u, r);
+    const long long b = A.rp[u], e = A.rp[u + 1];
+    int p = 0;
+    for (long long j0 = b; j0 < e; j0 += 32) {
+        const long long j = j0 + lane;
+        const int x = j < e ? head(A, j) : 0;
+        const bool k = j < e && keep(A, x);
+        const unsigned bal = __ballot_sync(0xffffffffu, k);
+        if (p + __popc(bal) > WARP_P) return false;
+        if (k) {
+            const int at = p + __popc(bal & ((1u << lane) - 1u));
+            ids[at] = x;
+            cis[at] = A.ci[x];
+        }
+        p += __popc(bal);
+    }
+    const int q = A.q;
+    if (p < q - 1) return true;
+    __syncwarp();
+    const int words = (p + 31) >> 5;
+    unsigned long long mine = 0;
+    for (int v = 0; v < p; v++) {
+        const int x = ids[v], cx = cis[v];
+        int t = 0;
+        for (int w = 0; w < words; w++) {
+            const int y = 32 * w + lane;
+            const unsigned bal = __ballot_sync(0xffffffffu, y < p && y != v && adjacent(A, x, cx, ids[y], cis[y]));
+            if (q == 3) t += __popc(bal);
+            else if (lane == 0) rows[v * WARP_STRIDE + w] = bal;
+        }
+        if (q == 3 && lane == 0) {
+            credit(A, x, (unsigned long long)t, r);
+            mine += (unsigned long long)t;
+        }
+    }
+    __syncwarp();
+    if (q > 3) {
+        for (int v = lane; v < p; v += 32) {
+            const unsigned long long t = cliques_of(q - 2, rows, WARP_STRIDE, words, v, 0, words);
+            credit(A, ids[v], t, r);
+            mine += t;
+        }
+    }
+    sum += mine;
+    __syncwarp();
+    return true;
+}
+
+// Cliques of every vertex (r < 0) or of the round's removed vertices, a warp
+// each; vertices with too many candidates are listed for the CTA launch.
+__device__ __forceinline__ void add_cliques(const TdsArgs &A, unsigned long long sum, int r) {
+    sum = warp_sum_u64(sum);
+    if ((threadIdx.x & 31) == 0 && sum) {
+        // every clique was counted once through each of its q - 1 members besides u
+        const unsigned long long k = sum / (unsigned long long)(A.q - 1);
+        atomicAdd((unsigned long long *)(r < 0 ? &A.ctl->f : &A.ctl->df), k);
+        // u's own weight matters in the initial counts only (it leaves in a round)
+    }
+}
+
+template <bool ROUND>
+__global__ void __launch_bounds__(WARP_TEAM) k_clq_warp(TdsArgs A) {
+    __shared__ int s_ids[WARP_TEAM / 32][WARP_P], s_cis[WARP_TEAM / 32][WARP_P];
+    __shared__ unsigned s_rows[WARP_TEAM / 32][WARP_P * WARP_STRIDE];
+    const TdsCtl *c = A.ctl;
+    if (ROUND && (c->status || c->error)) return;
+    const int r = ROUND ? (int)(c->round + 1) : -1;
+    const long long U = ROUND ? c->ucnt : A.n;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long W = (long long)gridDim.x * (WARP_TEAM / 32);
+    unsigned long long total = 0;
+    for (long long k = blockIdx.x * (long long)(WARP_TEAM / 32) + wid; k < U; k += W) {
+        const int u = ROUND ? A.front[k] : (int)k;
+        unsigned long long sum = 0;
+        if (!warp_vertex(A, u, r, s_ids[wid], s_cis[wid], s_rows[wid], sum)) {
+            if (lane == 0) A.big[atomicAdd(&A.ctl->nbig, 1)] = u;
+            __syncwarp();
+            continue;
+        }
+        sum = warp_sum_u64(sum);
+        if (!ROUND && lane == 0 && sum) atomicAdd((unsigned long long *)&A.w[u], sum / (unsigned long long)(A.q - 1));
+        if (lane == 0) total += sum;
+    }
+    add_cliques(A, total, r);
+}
+
 // positions of depth d (2 <= d <= QMAX - 1) start at pos_base(d): d of them,
 // one in the row of each member chosen before depth d
 __host__ __device__ constexpr int pos_base(int d) { return d * (d - 1) / 2 - 1; }
@@ -360,76 +492,118 @@ __device__ void clique_walk(const TdsArgs &A, int q, int u, long long j, long lo
     }
 }
 
-// every q-clique once, from its member u of lowest rank (degree, then id):
-// the lane of arc u -> v walks when v outranks u and keeps only members that
-// outrank u, so a hub lists just the cliques whose other members have higher
-// degree still, and the listing spreads over the low-degree vertices' warps
-__global__ void k_clq_count(TdsArgs A) {
-    const int lane = threadIdx.x & 31;
+
+// Vertices with more candidates than a warp takes, a CTA each.
+template <bool ROUND>
+__global__ void __launch_bounds__(CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
+    extern __shared__ int s_mem[];
+    __shared__ int s_cnt[CTA_TEAM / 32];
+    __shared__ unsigned long long s_sum;
+    constexpr int NW = CTA_TEAM / 32;
+    const TdsCtl *c = A.ctl;
+    if (ROUND && (c->status || c->error)) return;
+    const int r = ROUND ? (int)(c->round + 1) : -1;
+    const int nbig = c->nbig;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int q = A.q;
-    const long long W = (long long)gridDim.x * (blockDim.x >> 5);
-    long long cnt = 0;
-    for (long long u = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); u < A.n; u += W) {
+    const int cap = q == 3 ? CTA_P3 : CTA_P;
+    int *ids = s_mem, *cis = s_mem + cap;
+    unsigned *rows = (unsigned *)(cis + cap);
+    unsigned long long total = 0;
+    for (int k = blockIdx.x; k < nbig; k += gridDim.x) {
+        const int u = A.big[k];
+        const Keep keep(A, u, r);
         const long long b = A.rp[u], e = A.rp[u + 1];
-        const auto above = [&](int x) {
-            const long long dx = A.rp[x + 1] - A.rp[x];
-            return dx > e - b || (dx == e - b && x > (int)u);
-        };
-        for (long long j = b + lane; j < e; j += 32) {
-            const int v = head(A, j);
-            if (!above(v)) continue;
-            clique_walk(
-                A, q, (int)u, j, e, v, above,
-                [&](const int *c) {
-                    for (int t = 0; t < q; t++) atomicAdd((unsigned long long *)&A.w[c[t]], 1ull);
-                    cnt++;
+        __syncthreads();
+        if (tid == 0) s_sum = 0;
+        int p = 0;
+        for (long long j0 = b; j0 < e && p <= cap; j0 += CTA_TEAM) {  // candidates in id order
+            const long long j = j0 + tid;
+            const int x = j < e ? head(A, j) : 0;
+            const bool kp = j < e && keep(A, x);
+            const unsigned bal = __ballot_sync(0xffffffffu, kp);
+            __syncthreads();
+            if (lane == 0) s_cnt[wid] = __popc(bal);
+            __syncthreads();
+            int at = p, all = 0;
+            for (int o = 0; o < NW; o++) {
+                if (o < wid) at += s_cnt[o];
+                all += s_cnt[o];
+            }
+            at += __popc(bal & ((1u << lane) - 1u));
+            if (kp && at < cap) {
+                ids[at] = x;
+                cis[at] = A.ci[x];
+            }
+            p += all;
+        }
+        __syncthreads();
+        unsigned long long mine = 0;  // this thread's part of the cliques through each candidate
+        if (p > cap) {  // too many candidates for shared memory: walk the rows
+            for (long long j = b + tid; j < e; j += CTA_TEAM) {
+                const int v = head(A, j);
+                if (!keep(A, v)) continue;
+                clique_walk(A, q, u, j, e, v, [&](int x) { return keep(A, x); }, [&](const int *m) {
+                    mine += q - 1;
+                    for (int t = 1; t < q; t++) credit(A, m[t], 1, r);
                 });
+            }
+        } else if (p >= q - 1) {
+            const int words = (p + 31) >> 5, stride = words | 1;
+            for (int v = wid; v < p; v += NW) {
+                const int x = ids[v], cx = cis[v];
+                int t = 0;
+                for (int w = 0; w < words; w++) {
+                    const int y = 32 * w + lane;
+                    const unsigned bal = __ballot_sync(0xffffffffu, y < p && y != v && adjacent(A, x, cx, ids[y], cis[y]));
+                    if (q == 3) t += __popc(bal);
+                    else if (lane == 0) rows[(size_t)v * stride + w] = bal;
+                }
+                if (q == 3 && lane == 0) {
+                    credit(A, x, (unsigned long long)t, r);
+                    mine += (unsigned long long)t;
+                }
+            }
+            __syncthreads();
+            if (q > 3) {
+                for (int v = wid; v < p; v += NW) {  // lanes share the first member's words
+                    unsigned long long t = 0;
+                    for (int w = lane; w < words; w += 32) t += cliques_of(q - 2, rows, stride, words, v, w, w + 1);
+                    t = warp_sum_u64(t);
+                    if (lane == 0) {
+                        credit(A, ids[v], t, r);
+                        mine += t;
+                    }
+                }
+            }
+        }
+        mine = warp_sum_u64(mine);
+        if (lane == 0 && mine) atomicAdd(&s_sum, mine);
+        __syncthreads();
+        if (tid == 0) {
+            if (!ROUND && s_sum) atomicAdd((unsigned long long *)&A.w[u], s_sum / (unsigned long long)(q - 1));
+            total += s_sum;
         }
     }
-    for (int d = 16; d > 0; d >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, d);
-    if (lane == 0 && cnt) atomicAdd((unsigned long long *)&A.ctl->f, (unsigned long long)cnt);
+    if (wid == 0) add_cliques(A, total, r);
 }
 
-// the q-cliques of G[S_{i-1}] that die in round i (one warp per removed
-// vertex u): each is listed once, by its removed member of lowest rank
-// (degree, then id) -- u's walk keeps a member removed in this round only if
-// it outranks u -- and lowers f by one and each member outside U_i by one
-__global__ void k_clq_expand(TdsArgs A) {
-    const TdsCtl *ctl = A.ctl;
-    if (ctl->status || ctl->error) return;
-    const int r = (int)(ctl->round + 1);
-    const long long U = ctl->ucnt;
-    const int q = A.q;
-    const int lane = threadIdx.x & 31;
-    const long long W = (long long)gridDim.x * (blockDim.x >> 5);
-    long long dead = 0;
-    for (long long k = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); k < U; k += W) {
-        const int u = A.front[k];
-        const long long b = A.rp[u], e = A.rp[u + 1];
-        const auto keep = [&](int x) {
-            const int px = A.pr[x];
-            if (px < r) return false;  // left in an earlier round
-            if (px > r) return true;   // survives the round
-            const long long dx = A.rp[x + 1] - A.rp[x];
-            return dx > e - b || (dx == e - b && x > u);
-        };
-        for (long long j = b + lane; j < e; j += 32) {
-            const int v = head(A, j);
-            if (!keep(v)) continue;
-            clique_walk(A, q, u, j, e, v, keep, [&](const int *c) {
-                dead++;
-                for (int t = 1; t < q; t++)
-                    if (A.pr[c[t]] != r) atomicAdd((unsigned long long *)&A.w[c[t]], (unsigned long long)-1ll);
-            });
-        }
-    }
-    for (int d = 16; d > 0; d >>= 1) dead += __shfl_down_sync(0xffffffffu, dead, d);
-    if (lane == 0 && dead) atomicAdd((unsigned long long *)&A.ctl->df, (unsigned long long)dead);
+// ------------------------------------------------------------------ rounds
+
+__device__ __forceinline__ long long tds_floor(u128 x, u128 y) {
+    const u128 q = x / y;
+    return q > (u128)0x7fffffffffffffffULL ? 0x7fffffffffffffffLL : (long long)q;
 }
 
-__global__ void k_tds_close(TdsArgs A) {
+// ceil(x / y) - 1 (the largest integer strictly below x / y), -1 for x = 0
+__device__ __forceinline__ long long tds_below(u128 x, u128 y) {
+    if (x == 0) return -1;
+    return tds_floor(x - 1, y);
+}
+
+// f, |S|, the trace and the best prefix of the round just expanded
+__device__ void close_round(const TdsArgs &A) {
     TdsCtl *c = A.ctl;
-    if (c->status || c->error) return;
     if (c->ucnt == 0) {  // cannot happen (Lemma 4.2 / minimum rule)
         c->error = DUPIN_ERR_NO_PROGRESS;
         return;
@@ -451,8 +625,84 @@ __global__ void k_tds_close(TdsArgs A) {
         A.tr_size[i] = c->size;
         A.tr_peeled[i] = c->ucnt;
     }
-    c->minw = 0x7fffffffffffffffLL;
     if (c->size == 0) c->status = 1;
+}
+
+__device__ void plan_round(const TdsArgs &A) {
+    TdsCtl *c = A.ctl;
+    if (c->round + 1 > A.max_rounds) {
+        c->error = DUPIN_ERR_NO_PROGRESS;
+        return;
+    }
+    const u128 f = (u128)(unsigned long long)c->f, size = (u128)(unsigned long long)c->size;
+    const long long m = c->minw;
+    const long long below_g = tds_below(f, size);
+    if (A.lpo && c->round > 0 && m <= below_g) {  // Algorithm 4: some live w < g(S)
+        c->T = below_g > c->gpo_lt ? below_g : c->gpo_lt;
+        c->kind = 2;
+    } else {
+        long long T = tds_floor((u128)(unsigned long long)A.kD * f, (u128)(unsigned long long)A.D * size);
+        if (A.gpo) {  // Algorithm 3: tau_max refined at every main round
+            const u128 num = (u128)(unsigned long long)A.D * f, den = (u128)(unsigned long long)A.kD * size;
+            const long long le = tds_floor(num, den), lt = tds_below(num, den);
+            if (le > c->gpo_le) c->gpo_le = le;
+            if (lt > c->gpo_lt) c->gpo_lt = lt;
+            if (c->gpo_le > T) T = c->gpo_le;
+        }
+        c->kind = 0;
+        if (m > T) {  // the threshold selects nobody: the minimum rule
+            T = m;
+            c->kind = 1;
+        }
+        c->T = T;
+    }
+    c->ucnt = 0;
+    c->df = 0;
+    c->nbig = 0;
+}
+
+// the minimum live weight; the last block through closes the round (unless
+// none has run yet) and plans the next
+__global__ void k_tds_close(TdsArgs A, int first) {
+    TdsCtl *c = A.ctl;
+    if (c->status || c->error) return;
+    long long m = 0x7fffffffffffffffLL;
+    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < A.n; u += (long long)gridDim.x * blockDim.x)
+        if (A.pr[u] == DUPIN_LIVE && A.w[u] < m) m = A.w[u];
+    m = warp_min64(m);
+    if ((threadIdx.x & 31) == 0 && m != 0x7fffffffffffffffLL) atomicMin(&c->minw, m);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&c->blocks, 1) == (int)gridDim.x - 1) {
+        __threadfence();
+        c->blocks = 0;
+        c->minw = atomicMin(&c->minw, 0x7fffffffffffffffLL);  // read where the other blocks wrote
+        if (!first) close_round(A);
+        if (!c->status && !c->error) plan_round(A);
+        c->minw = 0x7fffffffffffffffLL;
+    }
+}
+
+__global__ void k_tds_select(TdsArgs A) {
+    const TdsCtl *c = A.ctl;
+    if (c->status || c->error) return;
+    const long long T = c->T;
+    const int r = (int)(c->round + 1);
+    const int lane = threadIdx.x & 31;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long b = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); b < A.n; b += stride) {
+        const long long u = b + lane;
+        const bool sel = u < A.n && A.pr[u] == DUPIN_LIVE && A.w[u] <= T;
+        const unsigned m = __ballot_sync(0xffffffffu, sel);
+        if (!m) continue;
+        long long base = 0;
+        if (lane == 0) base = (long long)atomicAdd((unsigned long long *)&A.ctl->ucnt, (unsigned long long)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (sel) {
+            A.pr[u] = r;
+            A.front[base + __popc(m & ((1u << lane) - 1u))] = (int)u;
+        }
+    }
 }
 
 __global__ void k_tds_mask(const int *pr, long long n, const TdsCtl *c, uint8_t *mask) {
@@ -461,7 +711,22 @@ __global__ void k_tds_mask(const int *pr, long long n, const TdsCtl *c, uint8_t 
         mask[u] = (long long)pr[u] > br ? 1 : 0;
 }
 
-__global__ void k_tds_minw_init(TdsCtl *c) { c->minw = 0x7fffffffffffffffLL; }
+// the CTA kernels' shared memory, once per device
+int set_clique_smem() {
+    static std::mutex mu;
+    static bool done[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return dupin_fail(DUPIN_ERR_CUDA, "device ordinal out of range");
+    std::lock_guard<std::mutex> lk(mu);
+    if (done[dev]) return DUPIN_OK;
+    for (const void *f : {(const void *)k_clq_cta<false>, (const void *)k_clq_cta<true>}) {
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CTA_SMEM);
+        if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncSetAttribute(k_clq_cta)");
+    }
+    done[dev] = true;
+    return DUPIN_OK;
+}
 
 }  // namespace
 
@@ -483,55 +748,63 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
     A.gpo = (p->flags & (DUPIN_GPO | DUPIN_LPO)) ? 1 : 0;
     A.lpo = (p->flags & DUPIN_LPO) ? 1 : 0;
     A.q = p->metric == DUPIN_KCLIDS ? p->clique_q : 3;
-    const bool tri = p->metric == DUPIN_TDS;  // the triangle kernels; kCLiDS (any q) walks
     A.max_rounds = max_rounds;
     A.tr_cap = tr_cap;
-    cudaError_t e = cudaSuccess;
-    void *buf[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    auto alloc = [&](int k, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMallocAsync(&buf[k], bytes ? bytes : 8, s);
+    int rc = set_clique_smem();
+    if (rc) return rc;
+    // one block from the graphs' pool (it keeps freed memory; the default pool
+    // would give it back to the driver at every call's end)
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        const size_t o = at;
+        at += (bytes + 255) & ~(size_t)255;
+        return o;
     };
-    alloc(0, 8 * (size_t)n);
-    alloc(1, 4 * (size_t)n);
-    alloc(2, 4 * (size_t)n);
-    alloc(3, sizeof(TdsCtl));
-    alloc(4, 8 * (size_t)tr_cap);
-    alloc(5, 8 * (size_t)tr_cap);
-    alloc(6, 8 * (size_t)tr_cap);
-    auto release = [&]() {
-        for (void *q : buf)
-            if (q) cudaFreeAsync(q, s);
-        cudaStreamSynchronize(s);
-    };
+    const size_t o_w = part(8 * (size_t)n), o_pr = part(4 * (size_t)n), o_front = part(4 * (size_t)n),
+                 o_big = part(4 * (size_t)n), o_ci = part(4 * (size_t)n), o_ctl = part(sizeof(TdsCtl)),
+                 o_trf = part(8 * (size_t)tr_cap), o_trs = part(8 * (size_t)tr_cap), o_trp = part(8 * (size_t)tr_cap),
+                 o_hist = part(4 * DEG_BINS), o_mask = part((size_t)n),
+                 o_bits = part(4 * (size_t)CORE_WORDS * (size_t)std::min<long long>(n, CORE_MAX));
+    unsigned char *buf = nullptr;
+    cudaError_t e = graph_pool_alloc((void **)&buf, at, s);
     if (e != cudaSuccess) {
-        release();
         cudaGetLastError();
         return dupin_fail(e == cudaErrorMemoryAllocation ? DUPIN_ERR_OOM : DUPIN_ERR_CUDA,
                           std::string("clique peel state: ") + cudaGetErrorString(e));
     }
-    A.w = (long long *)buf[0];
-    A.pr = (int *)buf[1];
-    A.front = (int *)buf[2];
-    A.ctl = (TdsCtl *)buf[3];
-    A.tr_f = (long long *)buf[4];
-    A.tr_size = (long long *)buf[5];
-    A.tr_peeled = (long long *)buf[6];
-    const int vgrid = sms * 8;
+    auto release = [&]() { graph_pool_free(buf, s); };
+    A.w = (long long *)(buf + o_w);
+    A.pr = (int *)(buf + o_pr);
+    A.front = (int *)(buf + o_front);
+    A.big = (int *)(buf + o_big);
+    A.ci = (int *)(buf + o_ci);
+    A.ctl = (TdsCtl *)(buf + o_ctl);
+    A.tr_f = (long long *)(buf + o_trf);
+    A.tr_size = (long long *)(buf + o_trs);
+    A.tr_peeled = (long long *)(buf + o_trp);
+    A.hist = (int *)(buf + o_hist);
+    A.bits = (unsigned *)(buf + o_bits);
+    // grids: as many blocks as there is work for, up to a few per SM
+    const int vgrid = (int)std::max<long long>(1, std::min<long long>(sms * 8, (n + 255) / 256));
+    const int cgrid = (int)std::max<long long>(1, std::min<long long>(sms, (n + 1023) / 1024));
+    const int wgrid = (int)std::max<long long>(1, std::min<long long>(sms * 8, (n + WARP_TEAM / 32 - 1) / (WARP_TEAM / 32)));
     k_tds_reset<<<vgrid, 256, 0, s>>>(A);
-    if (tri) k_tds_count<<<vgrid, 256, 0, s>>>(A);
-    else k_clq_count<<<vgrid, 256, 0, s>>>(A);
+    k_core_hist<<<vgrid, 256, 0, s>>>(A);
+    k_core_threshold<<<1, 1024, 0, s>>>(A);
+    k_core_rows<<<vgrid, 256, 0, s>>>(A);
+    k_core_bits<<<wgrid, WARP_TEAM, 0, s>>>(A);
+    k_clq_warp<false><<<wgrid, WARP_TEAM, 0, s>>>(A);
+    k_clq_cta<false><<<sms, CTA_TEAM, CTA_SMEM, s>>>(A);
     k_tds_start<<<1, 1, 0, s>>>(A);
-    k_tds_minw_init<<<1, 1, 0, s>>>(A.ctl);
+    k_tds_close<<<cgrid, 1024, 0, s>>>(A, 1);
     TdsCtl hc;
-    int rc = DUPIN_OK;
-    for (long long done_rounds = 0;; done_rounds += 32) {
-        for (int j = 0; j < 32; j++) {
-            k_tds_min<<<vgrid, 256, 0, s>>>(A);
-            k_tds_plan<<<1, 1, 0, s>>>(A);
+    int group = 2;
+    for (long long done_rounds = 0;; done_rounds += group, group = group < 32 ? 2 * group : 32) {
+        for (int j = 0; j < group; j++) {
             k_tds_select<<<vgrid, 256, 0, s>>>(A);
-            if (tri) k_tds_expand<<<vgrid, 256, 0, s>>>(A);
-            else k_clq_expand<<<vgrid, 256, 0, s>>>(A);
-            k_tds_close<<<1, 1, 0, s>>>(A);
+            k_clq_warp<true><<<wgrid, WARP_TEAM, 0, s>>>(A);
+            k_clq_cta<true><<<sms, CTA_TEAM, CTA_SMEM, s>>>(A);
+            k_tds_close<<<cgrid, 1024, 0, s>>>(A, 0);
         }
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, A.ctl, sizeof(hc), cudaMemcpyDeviceToHost, s);
@@ -564,13 +837,9 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
         const bool dev = (p->flags & DUPIN_RESULT_DEVICE) != 0;
         const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         if (r->best_mask && n > 0) {
-            uint8_t *mk = nullptr;
-            e = dev ? cudaSuccess : cudaMallocAsync((void **)&mk, (size_t)n, s);
-            if (e == cudaSuccess) {
-                k_tds_mask<<<sms * 4, 256, 0, s>>>(A.pr, n, A.ctl, dev ? r->best_mask : mk);
-                if (!dev) e = cudaMemcpyAsync(r->best_mask, mk, (size_t)n, cudaMemcpyDeviceToHost, s);
-                if (mk) cudaFreeAsync(mk, s);
-            }
+            uint8_t *mk = buf + o_mask;
+            k_tds_mask<<<vgrid, 256, 0, s>>>(A.pr, n, A.ctl, dev ? r->best_mask : mk);
+            if (!dev) e = cudaMemcpyAsync(r->best_mask, mk, (size_t)n, cudaMemcpyDeviceToHost, s);
         }
         if (e == cudaSuccess && r->peel_round && n > 0)
             e = cudaMemcpyAsync(r->peel_round, A.pr, 4 * (size_t)n, kind, s);
