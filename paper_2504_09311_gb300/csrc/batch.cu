@@ -1,14 +1,11 @@
 // batch.cu -- dupin_peel_batch: many independent graphs, one CTA per graph.
 //
 // A persistent grid pulls graphs from an atomic queue; each CTA runs a whole
-// peel (Algorithm 2, Sec. 4.1) of its graph: initial weights (a warp per row,
-// the whole CTA for rows longer than CTA_BIGROW), then the rounds.  The
-// graph's weights stay in global memory (L2-resident for window-sized
-// graphs) with the vertex state in the sign (w >= 0 live, w = -i removed in
-// round i); 64-vertex segment minima, double-buffered by round parity, sit in
-// shared memory, so a round scans only segments that can hold selected
-// vertices and every warp closes the round itself (two barriers per round),
-// exactly as the single-graph tail does.  Graphs with more than CTA_MAX_N
+// peel (Algorithm 2, Sec. 4.1) of its graph: initial weights, the first rounds
+// on the whole graph with its weights in global memory (w >= 0 live, w = -i
+// removed in round i; 64-vertex segment minima, double-buffered by round
+// parity, in shared memory), and, once the live set fits the CTA's shared
+// memory, the rounds of local_device.cuh.  Graphs with more than CTA_MAX_N
 // vertices take the single-graph path.  Results are identical to dupin_peel:
 // the arithmetic is the same exact integer peel.
 #include <cuda_runtime.h>
@@ -24,15 +21,19 @@
 #include <map>
 #include <mutex>
 #include "dupin_internal.h"
-#include "peel_device.cuh"
+#include "local_device.cuh"
 
-// Two launch shapes of the batched kernel, picked per device (default, or by
-// dupin_batch_tune): 128 threads x 4 CTAs per SM, or 256 threads x 2.
+// Launch shapes of the batched kernel, picked per device (default, or by
+// dupin_batch_tune): 128 threads x 4 CTAs per SM, or 256 threads x 2; a launch
+// of at most one graph per SM takes 256 threads x 1.
 #define CTA_MAX_SEG 2048
 #define CTA_MAX_N ((long long)CTA_MAX_SEG * TAIL_SEG)
 static_assert(CTA_MAX_N == DUPIN_BATCH_CTA_MAX_N, "header limit out of date");
 #define CTA_BIGROW 2048
 #define CTA_BIGLIST 64
+
+#define CTA_ILP 8    // arcs per thread in flight in a large round
+#define CTA_ROW 32  // rows of up to this many arcs are summed by one thread
 
 struct CtaJob {
     long long n, arcs;
@@ -41,8 +42,10 @@ struct CtaJob {
     const long long *cw;  // nullptr: DG
     const long long *a;   // nullptr: 0
     const int *hubs;      // heads of hub-coded arcs
+    long long n_hubs;
     long long kD, D, max_rounds;
     int use_min, gpo, lpo;
+    int pad;
     long long *w;      // [n] workspace
     int *front;        // [n] workspace
     int *pr;           // [n] output
@@ -53,10 +56,43 @@ struct CtaJob {
     long long *out;    // [8]: R, best round, best size, best f hi, best f lo, minimum-rule rounds, error, 0
 };
 
+// shared memory of one CTA besides the dynamic part
 template <int NT>
-__device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf, TailAcc<NT / 32> *s_acc, long long *s_w,
-                                             long long *s_pref, long long *s_fs, long long *s_fl, int *s_big,
-                                             int *s_nbig, unsigned long long *s_lo, unsigned long long *s_hi) {
+struct CtaShared {
+    TailAcc<NT / 32> acc[2];
+    long long w[NT / 32];
+    union {                    // a large round, per warp: 32 rows' first arcs and the arcs before each
+        struct {
+            long long start[NT];
+            int before[NT / 32][32];
+        };
+        unsigned rows[2 * NT];  // the same for the local rounds
+    };
+    int hubs[DUPIN_HUB_MAX];   // heads of hub-coded arcs
+    long long fs[TAIL_FAST], fl[TAIL_FAST];
+    unsigned long long lo[NT / 32], hi[NT / 32];
+    LocalHand hand;
+    int big[CTA_BIGLIST];
+    int nbig, nrows, next, job;
+    CtaJob J;
+};
+
+// One graph, one CTA.  The first rounds work on the whole graph, its weights in
+// global memory; once the live set is small enough for the CTA's shared memory
+// (at once, for a small graph) its vertex state moves there (local_device.cuh)
+// and the rounds go on over the graph's own rows, w holding each live vertex's
+// place.  On the largest window of the batched workload (75,000 vertices, 1,058
+// rounds) a round took 13 us: 1,172 segments to look over, weights and updates
+// in L2.  After five rounds 3,700 vertices are left.  (Copying the live arcs
+// out as well cost 2 ms of latency there, more than the dead arcs do; a matrix
+// as in dense.cu, 2.5-5 us per round in one CTA, its registers spilled.)
+// 61 windows of up to 500,000 edges: 14.6 -> 6.3 ms; 4,096: kernel 46.5 -> 27.3
+// ms, bound by the latency of dependent loads with 16 warps per SM (128
+// registers each; three CTAs per SM without spills: 30 ms).
+template <int NT>
+__device__ __forceinline__ void cta_peel_one(const CtaJob &J, unsigned char *smem, long long smem_bytes,
+                                             CtaShared<NT> &sh) {
+    constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const long long n = J.n;
     const bool dg = J.cw == nullptr;
@@ -64,46 +100,73 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
     const long long *rp = J.rp;
     const int *col = J.col;
     const long long *cw = J.cw;
-    const int *hubs = J.hubs;
+    const int *hubs = sh.hubs;
+    for (int h = tid; h < (int)J.n_hubs; h += NT) sh.hubs[h] = J.hubs[h];
+    long long *segbuf = (long long *)smem;
     const int nseg = (int)((n + TAIL_SEG - 1) / TAIL_SEG);
 
-    // ---- initial peeling weights w_u = a_u + sum_v c_uv (Sec. 2.2)
-    if (tid == 0) *s_nbig = 0;
+    // ---- initial peeling weights w_u = a_u + sum_v c_uv (Sec. 2.2): a thread
+    // per row of up to CTA_ROW arcs, a warp per longer one, the whole CTA for
+    // the longest (a warp per row throughout left most lanes idle and one
+    // row's latency per warp exposed: rows have 13 arcs on average)
+    if (tid == 0) {
+        sh.nbig = 0;
+        sh.nrows = 0;
+        sh.next = 0;
+    }
+    __syncthreads();
     for (long long u = tid; u < n; u += NT) {
-        const long long d = rp[u + 1] - rp[u];
-        w[u] = dg ? (d << 32) : (J.a ? J.a[u] : 0);
+        const long long b = rp[u], e = rp[u + 1];
+        long long x = dg ? (e - b) << 32 : (J.a ? J.a[u] : 0);
+        if (!dg) {
+            if (e - b <= CTA_ROW) {
+#pragma unroll 4
+                for (long long p = b; p < e; p++) x += cw[p];
+            } else {
+                J.front[atomicAdd(&sh.nrows, 1)] = (int)u;
+            }
+        }
+        w[u] = x;
     }
     __syncthreads();
     if (!dg) {
-        for (long long u = wid; u < n; u += (NT / 32)) {
+        const int nrows = sh.nrows;
+        for (;;) {
+            int k = 0;
+            if (lane == 0) k = atomicAdd(&sh.next, 1);
+            k = __shfl_sync(0xffffffffu, k, 0);
+            if (k >= nrows) break;
+            const int u = J.front[k];
             const long long b = rp[u], e = rp[u + 1];
             if (e - b > CTA_BIGROW) {
-                int k = 0;
+                int x = 0;
                 if (lane == 0) {
-                    k = atomicAdd(s_nbig, 1);
-                    if (k < CTA_BIGLIST) s_big[k] = (int)u;
+                    x = atomicAdd(&sh.nbig, 1);
+                    if (x < CTA_BIGLIST) sh.big[x] = u;
                 }
-                k = __shfl_sync(0xffffffffu, k, 0);
-                if (k < CTA_BIGLIST) continue;  // the whole CTA sums it below
+                x = __shfl_sync(0xffffffffu, x, 0);
+                if (x < CTA_BIGLIST) continue;  // the whole CTA sums it below
                 // list full: this warp sums the row itself
             }
             long long sum = 0;
+#pragma unroll 4
             for (long long p = b + lane; p < e; p += 32) sum += cw[p];
             sum = warp_sum64(sum);
             if (lane == 0) w[u] += sum;
         }
         __syncthreads();
-        const int nb = *s_nbig < CTA_BIGLIST ? *s_nbig : CTA_BIGLIST;
+        const int nb = sh.nbig < CTA_BIGLIST ? sh.nbig : CTA_BIGLIST;
         for (int k = 0; k < nb; k++) {
-            const long long u = s_big[k];
+            const long long u = sh.big[k];
             long long sum = 0;
+#pragma unroll 4
             for (long long p = rp[u] + tid; p < rp[u + 1]; p += NT) sum += cw[p];
             sum = warp_sum64(sum);
-            if (lane == 0) s_w[wid] = sum;
+            if (lane == 0) sh.w[wid] = sum;
             __syncthreads();
             if (tid == 0) {
                 long long t = 0;
-                for (int q = 0; q < (NT / 32); q++) t += s_w[q];
+                for (int q = 0; q < NW; q++) t += sh.w[q];
                 w[u] += t;
             }
             __syncthreads();
@@ -113,32 +176,40 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
     // f(V) = sum_u (w_u + a_u) / 2; segment minima of round 1
     {
         unsigned long long lo = 0, hi = 0;
+#pragma unroll 4
         for (long long u = tid; u < n; u += NT) {
             add128(lo, hi, (unsigned long long)w[u], 0);
             if (!dg && J.a) add128(lo, hi, (unsigned long long)J.a[u], 0);
         }
         warp_sum128(lo, hi);
         if (lane == 0) {
-            s_lo[wid] = lo;
-            s_hi[wid] = hi;
+            sh.lo[wid] = lo;
+            sh.hi[wid] = hi;
         }
     }
-    long long *first = segbuf + (1 & 1) * nseg;
-    for (int q = wid; q < nseg; q += (NT / 32)) {
-        const long long p = (long long)q * TAIL_SEG + 2 * lane;
-        const long long w0 = p < n ? w[p] : -1, w1 = p + 1 < n ? w[p + 1] : -1;
-        long long m = kMaxLL;
-        if (w0 >= 0) m = w0;
-        if (w1 >= 0 && w1 < m) m = w1;
-        m = warp_min64(m);
-        if (lane == 0) first[q] = m;
-    }
-    if (tid < 2) s_acc[tid].F = 0;
+    // every segment's minimum; returns the smallest that this warp found
+    auto minima = [&](long long *seg) -> long long {
+        long long all = kMaxLL;
+#pragma unroll 4
+        for (int q = wid; q < nseg; q += NW) {
+            const long long p = (long long)q * TAIL_SEG + 2 * lane;
+            const long long w0 = p < n ? w[p] : -1, w1 = p + 1 < n ? w[p + 1] : -1;
+            long long m = kMaxLL;
+            if (w0 >= 0) m = w0;
+            if (w1 >= 0 && w1 < m) m = w1;
+            m = warp_min64(m);
+            if (lane == 0) seg[q] = m;
+            all = m < all ? m : all;
+        }
+        return all;
+    };
+    minima(segbuf + nseg);
+    if (tid < 2) sh.acc[tid].F = 0;
     __syncthreads();
     RoundState st;
     {
         unsigned long long lo = 0, hi = 0;
-        for (int q = 0; q < (NT / 32); q++) add128(lo, hi, s_lo[q], s_hi[q]);
+        for (int q = 0; q < NW; q++) add128(lo, hi, sh.lo[q], sh.hi[q]);
         st.f = mk128(lo, hi) >> 1;
     }
     st.round = 0;
@@ -159,12 +230,73 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
         J.tr_peeled[0] = 0;
     }
     int err = 0;
-    // the round loop in two forms: NARROW (f < 2^62, so every sum of a
-    // round fits 64 bits: 64-bit adds, 32-bit warp reductions) or wide
+    LocalState S;
+    GraphArcs G = {nullptr, nullptr, col, hubs, cw, w};
+    long long nloc = 0;  // vertices whose state is in shared memory (0: not moved)
+    auto localise = [&]() {
+        const long long Ln = st.size;
+        unsigned *start = local_layout(S, smem, Ln, 8), *deg = start + Ln;
+        G.start = start;
+        G.deg = deg;
+        if (tid == 0) sh.nrows = 0;
+        __syncthreads();
+        for (int q = wid; q < nseg; q += NW) {
+            const long long p = (long long)q * TAIL_SEG + 2 * lane;
+            const long long w0 = p < n ? w[p] : -1, w1 = p + 1 < n ? w[p + 1] : -1;
+            const unsigned b0 = __ballot_sync(0xffffffffu, w0 >= 0), b1 = __ballot_sync(0xffffffffu, w1 >= 0);
+            if (!(b0 | b1)) continue;
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&sh.nrows, __popc(b0) + __popc(b1));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            const unsigned lt = (1u << lane) - 1u;
+            int slot = base + __popc(b0 & lt) + __popc(b1 & lt);
+            if (w0 >= 0) {  // its weight moves to its slot; its slot stands in its place
+                S.tw[slot] = w0;
+                J.front[slot] = (int)p;
+                w[p] = slot;
+                start[slot] = (unsigned)rp[p];
+                deg[slot++] = (unsigned)(rp[p + 1] - rp[p]);
+            }
+            if (w1 >= 0) {
+                S.tw[slot] = w1;
+                J.front[slot] = (int)(p + 1);
+                w[p + 1] = slot;
+                start[slot] = (unsigned)rp[p + 1];
+                deg[slot] = (unsigned)(rp[p + 2] - rp[p + 1]);
+            }
+        }
+        for (long long p = Ln + tid; p < (long long)S.nseg * TAIL_SEG; p += NT) S.tw[p] = -1;  // pads: gone
+        if (tid < 2) sh.acc[tid].F = 0;
+        S.kD = J.kD;
+        S.D = J.D;
+        S.max_rounds = J.max_rounds;
+        S.use_min = J.use_min;
+        S.gpo = J.gpo;
+        S.lpo = J.lpo;
+        S.tr_f_hi = J.tr_f_hi;
+        S.tr_f_lo = J.tr_f_lo;
+        S.tr_size = J.tr_size;
+        S.tr_peeled = J.tr_peeled;
+        S.tr_cap = J.tr_cap;
+        __syncthreads();
+        local_minima<NT>(S.tw, S.nseg, S.segbuf + ((st.round + 1) & 1) * S.nseg);
+        __syncthreads();
+        nloc = Ln;
+    };
+    // the rounds in two forms: NARROW (f < 2^62, so every sum of a round fits
+    // 64 bits: 64-bit adds, 32-bit warp reductions) or wide
     auto rounds = [&](auto narrow_tag) {
         constexpr bool NARROW = decltype(narrow_tag)::value;
-        TailRound R = tail_plan<NARROW>(J.kD, J.D, J.use_min, J.gpo, J.lpo, st, seg_global_min(first, nseg));
+        // live vertices whose state fits shared memory (rows' bounds are 32-bit)
+        long long fits = J.arcs < (1ll << 32) ? (smem_bytes - 1024) / 18 - 16 : 0;
+        fits -= fits / 64;  // the segments' minima
+        TailRound R = tail_plan<NARROW>(J.kD, J.D, J.use_min, J.gpo, J.lpo, st, seg_global_min(segbuf + nseg, nseg));
         while (!R.done) {
+            if (st.size <= fits) {
+                localise();
+                err = local_rounds<NT, NARROW>(S, G, st, sh.acc, sh.rows, &sh.hand);
+                return;
+            }
             if (R.i > J.max_rounds) {
                 err = DUPIN_ERR_NO_PROGRESS;
                 break;
@@ -172,7 +304,7 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
             const long long i = R.i;
             const long long *cur = segbuf + (i & 1) * nseg;
             long long *nxt = segbuf + ((i + 1) & 1) * nseg;
-            TailAcc<NT / 32> &acc = s_acc[i & 1];
+            TailAcc<NW> &acc = sh.acc[i & 1];
             // ---- select
             unsigned long long wlo = 0, whi = 0;
             long long mins = kMaxLL;  // new minimum over the segments this lane looked at
@@ -218,8 +350,8 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
                             else add128(wlo, whi, (unsigned long long)w0, 0);
                             J.front[slot] = (int)p;
                             if (slot < TAIL_FAST) {
-                                s_fs[slot] = rp[p];
-                                s_fl[slot] = rp[p + 1] - rp[p];
+                                sh.fs[slot] = rp[p];
+                                sh.fl[slot] = rp[p + 1] - rp[p];
                             }
                             slot++;
                         }
@@ -229,8 +361,8 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
                             else add128(wlo, whi, (unsigned long long)w1, 0);
                             J.front[slot] = (int)(p + 1);
                             if (slot < TAIL_FAST) {
-                                s_fs[slot] = rp[p + 1];
-                                s_fl[slot] = rp[p + 2] - rp[p + 1];
+                                sh.fs[slot] = rp[p + 1];
+                                sh.fl[slot] = rp[p + 2] - rp[p + 1];
                             }
                         }
                     }
@@ -238,65 +370,130 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
             }
             // the select's sums and minimum stay in registers until the expand's
             __syncthreads();
-            if (tid == 0) s_acc[(i + 1) & 1].F = 0;
+            if (tid == 0) sh.acc[(i + 1) & 1].F = 0;
             const int F = (int)acc.F;
-            // ---- expand: every arc of the frontier (heads read from global memory)
+            // ---- expand: every arc of the frontier (heads read from global
+            // memory), TAIL_ILP per thread in flight
             unsigned long long ilo = 0, ihi = 0;
             long long mind = kMaxLL;
-            auto arc = [&](long long pos) {
-                const int v = arc_head(col[pos], hubs);
-                const long long c = dg ? DUPIN_Q_ONE : cw[pos];
-                const long long wv = w[v];
-                if (wv >= 0) {
-                    const long long old = (long long)atomicAdd((unsigned long long *)&w[v], (unsigned long long)(-c));
-                    atomicMin(&nxt[v / TAIL_SEG], old - c);
-                    mind = old - c < mind ? old - c : mind;
-                } else if (wv == -i) {
-                    if (NARROW) ilo += (unsigned long long)c;
-                    else add128(ilo, ihi, (unsigned long long)c, 0);
+            auto arcs = [&](const long long (&pos)[TAIL_ILP]) {
+                int v[TAIL_ILP];
+                long long c[TAIL_ILP], wv[TAIL_ILP], nv[TAIL_ILP];
+#pragma unroll
+                for (int u = 0; u < TAIL_ILP; u++) {
+                    if (pos[u] >= 0) {
+                        v[u] = arc_head(col[pos[u]], hubs);
+                        c[u] = dg ? DUPIN_Q_ONE : cw[pos[u]];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < TAIL_ILP; u++) wv[u] = pos[u] >= 0 ? w[v[u]] : -i - 1;
+#pragma unroll
+                for (int u = 0; u < TAIL_ILP; u++) {
+                    nv[u] = kMaxLL;
+                    if (wv[u] >= 0) {
+                        nv[u] = (long long)atomicAdd((unsigned long long *)&w[v[u]], (unsigned long long)(-c[u])) - c[u];
+                    } else if (wv[u] == -i) {
+                        if (NARROW) ilo += (unsigned long long)c[u];
+                        else add128(ilo, ihi, (unsigned long long)c[u], 0);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < TAIL_ILP; u++) {
+                    if (wv[u] >= 0 && nv[u] < nxt[v[u] / TAIL_SEG]) atomicMin(&nxt[v[u] / TAIL_SEG], nv[u]);  // minima only fall here
+                    mind = nv[u] < mind ? nv[u] : mind;
                 }
             };
             if (F <= TAIL_FAST) {
                 // chunks of 32 consecutive arcs of one vertex, chunk c to warp
-                // c % (NT / 32); the walk is the same in every lane of a warp
+                // c % NW; the walk is the same in every lane of a warp
                 int e = 0;
                 long long cbase = 0, c = wid;
-                long long a0 = F > 0 ? s_fs[0] : 0, ln = F > 0 ? s_fl[0] : 0;
+                long long a0 = F > 0 ? sh.fs[0] : 0, ln = F > 0 ? sh.fl[0] : 0;
                 while (e < F) {
-                    if (c >= cbase + ((ln + 31) >> 5)) {
-                        cbase += (ln + 31) >> 5;
-                        e++;
-                        if (e < F) {
-                            a0 = s_fs[e];
-                            ln = s_fl[e];
+                    long long pos[TAIL_ILP];
+#pragma unroll
+                    for (int u = 0; u < TAIL_ILP; u++) {
+                        pos[u] = -1;
+                        while (e < F && c >= cbase + ((ln + 31) >> 5)) {
+                            cbase += (ln + 31) >> 5;
+                            e++;
+                            if (e < F) {
+                                a0 = sh.fs[e];
+                                ln = sh.fl[e];
+                            }
                         }
-                        continue;
+                        if (e < F) {
+                            const long long off = (c - cbase) * 32 + lane;
+                            if (off < ln) pos[u] = a0 + off;
+                            c += NW;
+                        }
                     }
-                    const long long off = (c - cbase) * 32 + lane;
-                    if (off < ln) arc(a0 + off);
-                    c += NT / 32;
+                    arcs(pos);
                 }
             } else {
-                for (int c0 = 0; c0 < F; c0 += NT) {
-                    const int qq = c0 + tid;
-                    long long deg = 0;
-                    if (qq < F) {
-                        const int p = J.front[qq];
-                        deg = rp[p + 1] - rp[p];
+                // Many vertices: each warp takes 32 rows at a time and spreads
+                // their arcs over its lanes, without block barriers; decrements
+                // return nothing, and the segments' minima are found anew by a
+                // pass over the weights (a returning atomic and a shared-memory
+                // minimum per arc took as long again as the loads).
+                long long *rs = sh.start + 32 * wid;
+                int *rb = sh.before[wid];
+                for (int g0 = 32 * wid; g0 < F; g0 += NT) {
+                    int deg = 0;
+                    if (g0 + lane < F) {
+                        const int p = J.front[g0 + lane];
+                        const long long b = rp[p];
+                        deg = (int)(rp[p + 1] - b);
+                        rs[lane] = b;
                     }
-                    long long tot;
-                    long long ex = block_excl_scan<NT / 32>(deg, s_w, tot);
-                    s_pref[tid] = ex;
-                    const int nq = (F - c0) < NT ? (F - c0) : NT;
-                    if (tid == 0) s_pref[nq] = tot;
-                    __syncthreads();
-                    for (long long x = tid; x < tot; x += NT) {
-                        const int e = smem_last_le(s_pref, nq, x);
-                        const int p = J.front[c0 + e];
-                        arc(rp[p] + (x - s_pref[e]));
+                    int incl = deg;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+                        if (lane >= d) incl += o;
                     }
-                    __syncthreads();
+                    rb[lane] = incl - deg;
+                    const int tot = __shfl_sync(0xffffffffu, incl, 31);
+                    __syncwarp();
+                    for (int x0 = lane; x0 - lane < tot; x0 += 32 * CTA_ILP) {
+                        int v[CTA_ILP];
+                        long long c[CTA_ILP], wv[CTA_ILP];
+#pragma unroll
+                        for (int u = 0; u < CTA_ILP; u++) {
+                            const int x = x0 + 32 * u;
+                            int t = 0;  // the last row that starts at or before x
+#pragma unroll
+                            for (int step = 16; step > 0; step >>= 1)
+                                if (rb[t + step] <= x) t += step;
+                            v[u] = 0;
+                            c[u] = 0;
+                            if (x < tot) {
+                                const long long pos = rs[t] + (x - rb[t]);
+                                v[u] = col[pos];
+                                c[u] = dg ? DUPIN_Q_ONE : cw[pos];
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < CTA_ILP; u++) {
+                            if (v[u] < 0) v[u] = hubs[-v[u] - 1];
+                            wv[u] = x0 + 32 * u < tot ? w[v[u]] : -i - 1;
+                        }
+#pragma unroll
+                        for (int u = 0; u < CTA_ILP; u++) {
+                            if (wv[u] >= 0) {
+                                atomicAdd((unsigned long long *)&w[v[u]], (unsigned long long)(-c[u]));
+                            } else if (wv[u] == -i) {
+                                if (NARROW) ilo += (unsigned long long)c[u];
+                                else add128(ilo, ihi, (unsigned long long)c[u], 0);
+                            }
+                        }
+                    }
+                    __syncwarp();
                 }
+                __syncthreads();
+                mind = minima(nxt);
+                mins = mind;
             }
             if (NARROW) {
                 if (__any_sync(0xffffffffu, wlo != 0)) wlo = warp_sum64_redux(wlo);
@@ -317,7 +514,7 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
             // ---- every warp: close round i, plan round i + 1
             u128 wsel, internal;
             long long mins_all;
-            tail_acc_sum<NT / 32, NARROW>(acc, wsel, internal, mins_all);
+            tail_acc_sum<NW, NARROW>(acc, wsel, internal, mins_all);
             st.f = st.f - (wsel - (internal >> 1));
             st.size -= F;
             st.round = i;
@@ -344,11 +541,14 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
     if ((unsigned long long)(st.f >> 64) == 0 && (unsigned long long)st.f < (1ull << 62)) rounds(std::true_type{});
     else rounds(std::false_type{});
     __syncthreads();
+    for (long long k = tid; k < nloc; k += NT) w[J.front[k]] = S.tw[k];
+    __syncthreads();
+#pragma unroll 4
     for (long long u = tid; u < n; u += NT) {
         const long long wv = w[u];
         J.pr[u] = wv < 0 ? (int)(-wv) : 0x7fffffff;
     }
-    if (tid == 0) {
+    if (tid == (NW - 1) * 32) {  // the local rounds keep the best prefix in the last warp
         J.out[0] = st.round;
         J.out[1] = st.best_round;
         J.out[2] = st.best_size;
@@ -361,41 +561,38 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, long long *segbuf,
 }
 
 template <int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_peel_cta(const CtaJob *jobs, int njobs, int *next) {
-    extern __shared__ __align__(16) long long s_seg[];  // 2 * CTA_MAX_SEG
-    __shared__ TailAcc<NT / 32> s_acc[2];
-    __shared__ long long s_w[(NT / 32)];
-    __shared__ long long s_pref[NT + 1];
-    __shared__ long long s_fs[TAIL_FAST], s_fl[TAIL_FAST];
-    __shared__ int s_big[CTA_BIGLIST];
-    __shared__ int s_nbig;
-    __shared__ unsigned long long s_lo[(NT / 32)], s_hi[(NT / 32)];
-    __shared__ int s_job;
+__global__ void __launch_bounds__(NT, MINB) k_peel_cta(const CtaJob *jobs, int njobs, int *next, int smem_bytes) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ CtaShared<NT> sh;
     for (;;) {
-        if (threadIdx.x == 0) s_job = atomicAdd(next, 1);
+        if (threadIdx.x == 0) sh.job = atomicAdd(next, 1);
         __syncthreads();
-        const int j = s_job;
-        __syncthreads();
+        const int j = sh.job;
         if (j >= njobs) break;
-        const CtaJob J = jobs[j];
-        const int nseg = (int)((J.n + TAIL_SEG - 1) / TAIL_SEG);
-        (void)nseg;
-        cta_peel_one<NT>(J, s_seg, s_acc, s_w, s_pref, s_fs, s_fl, s_big, &s_nbig, s_lo, s_hi);
+        static_assert(sizeof(CtaJob) % 8 == 0 && sizeof(CtaJob) / 8 <= NT, "a word per thread");
+        if (threadIdx.x < sizeof(CtaJob) / 8) ((long long *)&sh.J)[threadIdx.x] = ((const long long *)&jobs[j])[threadIdx.x];
+        __syncthreads();
+        cta_peel_one<NT>(sh.J, s_dyn, smem_bytes, sh);
         __syncthreads();
     }
 }
 
 // the launch shapes: threads per CTA, CTAs per SM the kernel is bounded for
 struct CtaShape {
-    int threads;
+    int threads, per_sm;
     const void *fn;
 };
-static const CtaShape kCtaShapes[2] = {{128, (const void *)k_peel_cta<128, 4>}, {256, (const void *)k_peel_cta<256, 2>}};
+static const CtaShape kCtaShapes[3] = {{128, 4, (const void *)k_peel_cta<128, 4>},
+                                       {256, 2, (const void *)k_peel_cta<256, 2>},
+                                       {256, 1, (const void *)k_peel_cta<256, 1>}};
+#define CTA_TUNED_SHAPES 2  // the autotuner's; the third is for launches of at most one graph per SM
 // Per device: the shape of launches with more graphs than one wave of the
 // widest shape holds ('large', tuned or default), or one shape for every
 // launch ('forced').  A launch that fits one wave of 256-thread CTAs leaves
 // SMs idle with either shape, so it takes the wider CTAs, which finish each
-// graph sooner (the serving case: few requests per launch).
+// graph sooner (the serving case: few requests per launch); one that fits one
+// CTA per SM takes the shape with all of the SM's registers and shared memory
+// (the 500,000-edge window: 6.2 ms against 7.8 ms at two per SM).
 struct ShapeSel {
     int large = 0;
     bool forced = false;
@@ -414,18 +611,35 @@ static int cta_shape_for(int dev, size_t njobs, int sms) {
     if (t_tune_shape >= 0) return t_tune_shape;
     const ShapeSel sel = shape_sel(dev);
     if (sel.forced) return sel.large;
+    if (njobs <= (size_t)sms) return 2;
     return njobs <= (size_t)2 * sms ? 1 : sel.large;
 }
 
-static int set_cta_smem() {
-    static bool done = false;
-    if (done) return DUPIN_OK;
-    for (const CtaShape &c : kCtaShapes) {
-        cudaError_t e = cudaFuncSetAttribute(c.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(2 * CTA_MAX_SEG * sizeof(long long)));
+// each shape's dynamic shared memory: what its CTAs per SM leave of the SM
+// (never less than the segment minima of the largest graph take), per device
+static int set_cta_smem(int shape, int *bytes) {
+    static std::mutex mu;
+    static int got[64][3] = {{0}};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return dupin_fail(DUPIN_ERR_CUDA, "device ordinal out of range");
+    std::lock_guard<std::mutex> lk(mu);
+    if (got[dev][shape] == 0) {
+        const CtaShape &c = kCtaShapes[shape];
+        int sm = 0, block = 0, reserved = 0;
+        cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+        cudaFuncAttributes fa;
+        cudaError_t e = cudaFuncGetAttributes(&fa, c.fn);
+        if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncGetAttributes(k_peel_cta)");
+        int dyn = std::min(sm / c.per_sm - reserved, block) - (int)fa.sharedSizeBytes;
+        dyn = std::max(dyn & ~1023, (int)(2 * CTA_MAX_SEG * sizeof(long long)));
+        e = cudaFuncSetAttribute(c.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
         if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncSetAttribute(k_peel_cta)");
+        got[dev][shape] = dyn;
     }
-    done = true;
+    *bytes = got[dev][shape];
     return DUPIN_OK;
 }
 
@@ -446,7 +660,7 @@ long long cta_job_bytes(const dupin_graph *g, const dupin_params *p) {
 }
 
 struct CtaBatch {
-    unsigned char *arena = nullptr;
+    unsigned char *arena = nullptr;  // from the graphs' pool, which keeps freed memory
     size_t nj = 0, outs_base = 0;
     std::vector<size_t> off_pr, off_tr;
     std::vector<long long> trcap;
@@ -456,14 +670,26 @@ struct CtaBatch {
     dupin_result *results = nullptr;
 };
 
+static bool wants_trace(const dupin_result &r) {
+    return r.trace_f_hi || r.trace_f_lo || r.trace_size || r.trace_peeled;
+}
+
 // Enqueue one persistent launch for graphs[idx[k]] on stream s (no host
 // synchronisation).  Results stay in the arena until cta_batch_finish.
 int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, dupin_result *results,
                       const std::vector<int64_t> &idx, cudaStream_t s, CtaBatch **out) {
     *out = nullptr;
     if (idx.empty()) return DUPIN_OK;
-    int rc = set_cta_smem();
+    int sms = 0, dev = 0, occ = 0, dyn = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int shape_id = cta_shape_for(dev, idx.size(), sms);
+    const CtaShape &shape = kCtaShapes[shape_id];
+    int rc = set_cta_smem(shape_id, &dyn);
     if (rc) return rc;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shape.fn, shape.threads, (size_t)dyn);
+    if (occ < 1) occ = 1;
+    const int grid = (int)std::min<long long>((long long)idx.size(), (long long)sms * occ);
     CtaBatch *B = new CtaBatch();
     B->graphs = graphs;
     B->params = params;
@@ -481,17 +707,22 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
     for (size_t k = 0; k < nj; k++) {
         const dupin_graph *g = graphs[idx[k]];
         const long long n = g->n;
-        B->trcap[k] = trace_cap_of(g, params[idx[k]]);
+        B->trcap[k] = wants_trace(results[idx[k]]) ? trace_cap_of(g, params[idx[k]]) : 0;
         off_w[k] = at;
         at = align256(at + 8 * (size_t)n);
         off_f[k] = at;
         at = align256(at + 4 * (size_t)n);
-        B->off_pr[k] = at;
-        at = align256(at + 4 * (size_t)n);
         B->off_tr[k] = at;
         at = align256(at + 32 * (size_t)B->trcap[k]);
     }
-    cudaError_t e = cudaMallocAsync((void **)&B->arena, at, s);
+    // peel rounds end to end, in the callers' order: adjacent result buffers
+    // are then copied back together
+    for (size_t k = 0; k < nj; k++) {
+        B->off_pr[k] = at;
+        at += 4 * (size_t)graphs[idx[k]]->n;
+    }
+    at = align256(at);
+    cudaError_t e = graph_pool_alloc((void **)&B->arena, at, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete B;
@@ -512,12 +743,14 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
         J.cw = dgr.cw;
         J.a = dgr.a;
         J.hubs = dgr.hubs;
+        J.n_hubs = dgr.n_hubs;
         J.kD = (long long)p.k_mult * (p.eps_den + p.eps_num);
         J.D = p.eps_den;
         J.max_rounds = p.max_rounds > 0 ? p.max_rounds : g->n + 1;
         J.use_min = J.kD < 2 * J.D ? 1 : 0;
         J.gpo = (p.flags & (DUPIN_GPO | DUPIN_LPO)) ? 1 : 0;
         J.lpo = (p.flags & DUPIN_LPO) ? 1 : 0;
+        J.pad = 0;
         J.w = (long long *)(arena + off_w[k]);
         J.front = (int *)(arena + off_f[k]);
         const bool dev = (p.flags & DUPIN_RESULT_DEVICE) != 0;
@@ -546,23 +779,16 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
         jobs.swap(sorted);
     }
     int *next = (int *)(arena + align256(sizeof(CtaJob) * nj));
-    int sms = 0, dev = 0, occ = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const CtaShape &shape = kCtaShapes[cta_shape_for(dev, nj, sms)];
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, shape.fn, shape.threads, 2 * CTA_MAX_SEG * sizeof(long long));
-    if (occ < 1) occ = 1;
-    const int grid = (int)std::min<long long>((long long)nj, (long long)sms * occ);
     e = cudaMemcpyAsync(arena, jobs.data(), sizeof(CtaJob) * nj, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, sizeof(int), s);
     if (e == cudaSuccess) {
         const CtaJob *jobs_dev = (const CtaJob *)arena;
         int njobs = (int)nj;
-        void *args[] = {(void *)&jobs_dev, (void *)&njobs, (void *)&next};
-        e = cudaLaunchKernel(shape.fn, dim3(grid), dim3(shape.threads), args, 2 * CTA_MAX_SEG * sizeof(long long), s);
+        void *args[] = {(void *)&jobs_dev, (void *)&njobs, (void *)&next, (void *)&dyn};
+        e = cudaLaunchKernel(shape.fn, dim3(grid), dim3(shape.threads), args, (size_t)dyn, s);
     }
     if (e != cudaSuccess) {
-        cudaFreeAsync(B->arena, s);
+        graph_pool_free(B->arena, s);
         delete B;
         return dupin_cuda_fail(e, "batched peel launch");
     }
@@ -582,6 +808,14 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
     int status = DUPIN_OK;
     std::string msg;
     if (per_job_status) per_job_status->assign(nj, DUPIN_OK);
+    // peel rounds waiting to be copied: adjacent in the arena and at the caller
+    char *run_to = nullptr;
+    const char *run_from = nullptr;
+    size_t run_bytes = 0;
+    auto flush = [&]() {
+        if (run_bytes && e == cudaSuccess) e = cudaMemcpyAsync(run_to, run_from, run_bytes, cudaMemcpyDeviceToHost, s);
+        run_bytes = 0;
+    };
     for (size_t k = 0; k < nj && e == cudaSuccess; k++) {
         const int64_t j = B->idx[k];
         const dupin_graph *g = B->graphs[j];
@@ -610,9 +844,16 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
         const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         const long long n = g->n;
         const int *pr_dev = dev && r.peel_round ? r.peel_round : (const int *)(arena + B->off_pr[k]);
-        if (r.peel_round && !dev && n > 0) e = cudaMemcpyAsync(r.peel_round, pr_dev, 4 * (size_t)n, kind, s);
+        if (r.peel_round && !dev && n > 0) {
+            if (run_bytes && ((char *)r.peel_round != run_to + run_bytes || (const char *)pr_dev != run_from + run_bytes)) flush();
+            if (!run_bytes) {
+                run_to = (char *)r.peel_round;
+                run_from = (const char *)pr_dev;
+            }
+            run_bytes += 4 * (size_t)n;
+        }
         const long long nt = o[0] + 1;
-        const bool want_tr = r.trace_f_hi || r.trace_f_lo || r.trace_size || r.trace_peeled;
+        const bool want_tr = wants_trace(r);
         const bool user_tr = dev && r.trace_f_hi && r.trace_f_lo && r.trace_size && r.trace_peeled;
         if (want_tr && !user_tr && e == cudaSuccess) {
             const long long cnt = std::min<long long>(nt, (long long)r.trace_cap);
@@ -636,7 +877,8 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
             if (dev) {
                 launch_mask(pr_dev, n, o[1], r.best_mask, s);
             } else {
-                e = cudaStreamSynchronize(s);
+                flush();
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
                 std::vector<int> tmp;
                 const int *prh = r.peel_round;
                 if (!prh) {
@@ -648,8 +890,9 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
             }
         }
     }
+    flush();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(arena, s);
+    graph_pool_free(arena, s);
     delete B;
     if (e != cudaSuccess) return dupin_cuda_fail(e, "batched peel");
     if (status) return dupin_fail(status, msg);
@@ -891,7 +1134,7 @@ extern "C" int dupin_batch_tune(dupin_graph *const *graphs, const dupin_params *
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaGetDevice");
     std::vector<dupin_result> res(gs.size());
-    const int nshape = (int)(sizeof(kCtaShapes) / sizeof(kCtaShapes[0]));
+    const int nshape = CTA_TUNED_SHAPES;
     std::vector<double> best(nshape, 1e300);
     int rc = DUPIN_OK;
     for (int rep = 0; rep < 3 && rc == DUPIN_OK; rep++) {

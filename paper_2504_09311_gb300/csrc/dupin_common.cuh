@@ -32,6 +32,10 @@ typedef unsigned __int128 u128;
 // its sub-graph has at most this many arcs (one SM fetches them); larger
 // ones go to the cluster tail.
 #define DUPIN_ONE_CTA_ARCS (1LL << 20)
+// ... and to the dense tail, where it fits, from this many arcs on: its round
+// takes 1.0 us, the one-CTA tail's 1.4 us and up (2.2 us at 830,000 arcs over
+// 5,000 vertices), but its build costs four launches and the matrix
+#define DUPIN_DENSE_ARCS (1LL << 16)
 // ... provided its live sub-graph fits the tail's arc buffer (2^27 arcs)
 #define DUPIN_TAIL_BUF_ARCS (1LL << 27)
 // On graphs of at least this many arcs the cluster tail gives the peel back to
@@ -172,6 +176,7 @@ struct PeelArgs {
     // most live vertices whose matrix fits there (0: no dense tail)
     void *dmat;
     int desz, dshift;
+    long long tail_smem;  // dynamic shared memory of the one-CTA tail
     int again;          // the cluster tail may give a collapsing graph back to the grid-wide rounds
     long long dcap;
 };
@@ -188,6 +193,7 @@ __host__ __device__ __forceinline__ long long dense_slice(long long L, int C) {
 
 // the tail that takes 'size' live vertices with 'arcs' live arcs
 __host__ __device__ __forceinline__ int tail_status(const PeelArgs &A, long long size, long long arcs) {
+    if (size <= A.dcap && arcs >= DUPIN_DENSE_ARCS) return ST_DENSE;
     if (size <= A.tail_cap && arcs <= A.one_arcs) return ST_TAIL;
     return size <= A.dcap ? ST_DENSE : ST_CLUSTER;
 }

@@ -82,6 +82,14 @@ struct PeelPlan {
 };
 
 DevGraph dev_graph(const dupin_graph *g, int metric);
+
+// A dense matrix's element for weights whose or is 'o': bytes (1, 4 or 8) and
+// the common low zero bits left out.
+inline void dense_element(unsigned long long o, int *esz, int *shift) {
+    *shift = o ? __builtin_ctzll(o) : 0;
+    *esz = (o >> *shift) >> 32 ? 8 : ((o >> *shift) >> 8 ? 4 : 1);
+    if (*esz == 8) *shift = 0;
+}
 long long workspace_bytes(long long n, long long arcs, bool has_cw, const PeelPlan &plan, int grid);
 PeelWorkspace *workspace_create(long long n, long long arcs, bool has_cw, const PeelPlan &plan, bool async,
                                 cudaStream_t s, int *rc);

@@ -38,6 +38,7 @@
 #include <mutex>
 
 #include "dupin_internal.h"
+#include "local_device.cuh"
 #include "peel_device.cuh"
 
 
@@ -1043,37 +1044,33 @@ __global__ void k_tail_grp(PeelArgs A) {
     }
 }
 
-// One CTA finishes the peel on the live sub-graph held in shared memory.
-// tw[p] is the peeling weight of local vertex p while it is live (>= 0) and
-// -i once it left in round i.  The live vertices are grouped in segments of
-// 64 with an exact minimum per segment, kept in two buffers by round parity:
-// round i reads its thresholds from one buffer and writes the new minima to
-// the other (recomputed for segments that lose vertices, lowered by
-// atomicMin on every decrement).  A round scans only segments that can hold
-// selected vertices, expands the frontier's arcs (from L2) with shared-memory
-// atomics, and then every warp closes the round and plans the next one
-// itself from the same shared data: two block barriers per round.
-// NARROW: f < 2^62 and the best f < 2^64 when the tail starts, so every sum
-// a round forms (at most 2f) fits 64 bits; the sums then take 64-bit adds
-// and 32-bit warp reductions, the products 64 x 64 -> 128-bit multiplies.
+// One CTA finishes the peel on the live sub-graph held in shared memory (the
+// rounds: local_device.cuh).  Where the sub-graph's arcs fit the rest of the
+// dynamic shared memory they are copied there too.
 template <bool NARROW>
 __device__ __forceinline__ void peel_tail_body(const PeelArgs &A, unsigned char *smem, TailAcc<TAIL_WARPS> *s_acc,
-                                               long long *s_w, long long *s_pref) {
+                                               unsigned *s_rows, LocalHand *s_hand) {
     PeelCtl *ctl = A.ctl;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x;
     const long long L = ctl->live_len;
-    const int nseg = (int)((L + TAIL_SEG - 1) / TAIL_SEG);
-    const long long LP = (long long)nseg * TAIL_SEG;
-    long long *tw = (long long *)smem;                                  // [LP]
-    long long *segbuf = (long long *)(smem + 8 * LP);                   // [2 nseg]
-    int *toff = (int *)(smem + 8 * LP + 16 * nseg);                     // [L+1]
-    unsigned short *tf = (unsigned short *)(smem + 8 * LP + 16 * nseg + 4 * (L + 1));  // [L]
     const int *live = ctl->live_sel ? A.live1 : A.live0;
-    const bool dg = A.tcw == nullptr;
-    const int *tcol = A.tcol;
-    const long long *tcw = A.tcw;
+    LocalState S;
+    int *toff = (int *)local_layout(S, smem, L, 4);
+    LocalArcs G = {toff, A.tcol, A.tcw};
+    const long long LP = (long long)S.nseg * TAIL_SEG;
+    S.kD = A.kD;
+    S.D = A.D;
+    S.max_rounds = A.max_rounds;
+    S.use_min = A.use_min;
+    S.gpo = A.gpo;
+    S.lpo = A.lpo;
+    S.tr_f_hi = A.tr_f_hi;
+    S.tr_f_lo = A.tr_f_lo;
+    S.tr_size = A.tr_size;
+    S.tr_peeled = A.tr_peeled;
+    S.tr_cap = A.tr_cap;
 
-    RoundState st;  // identical in every thread
+    RoundState st;  // identical in every thread (the best prefix in the last warp only)
     st.round = ctl->round;
     st.size = ctl->size;
     st.f = mk128(ctl->f_lo, ctl->f_hi);
@@ -1087,249 +1084,20 @@ __device__ __forceinline__ void peel_tail_body(const PeelArgs &A, unsigned char 
     st.n_min_rule = ctl->n_min_rule;
     st.scan = ctl->scan_volume;
     for (long long p = tid; p <= L; p += TAIL_THREADS) toff[p] = (int)A.tlrp[p];
-    for (long long p = tid; p < LP; p += TAIL_THREADS) tw[p] = p < L ? A.w[live[p]] : -1;  // pads: gone
+    for (long long p = tid; p < LP; p += TAIL_THREADS) S.tw[p] = p < L ? A.w[live[p]] : -1;  // pads: gone
     if (tid < 2) s_acc[tid].F = 0;
+    local_stage<TAIL_THREADS>(G, smem, local_bytes(L, 4), A.tail_smem, A.tlrp[L]);
     __syncthreads();
     // round i reads the minima in buffer (i & 1): fill the first round's buffer
-    long long *first = segbuf + ((st.round + 1) & 1) * nseg;
-    for (int q = wid; q < nseg; q += TAIL_WARPS) {
-        const longlong2 v = *(const longlong2 *)&tw[(long long)q * TAIL_SEG + 2 * lane];
-        long long m = kMaxLL;
-        if (v.x >= 0) m = v.x;
-        if (v.y >= 0 && v.y < m) m = v.y;
-        m = warp_min64(m);
-        if (lane == 0) first[q] = m;
-    }
+    local_minima<TAIL_THREADS>(S.tw, S.nseg, S.segbuf + ((st.round + 1) & 1) * S.nseg);
     __syncthreads();
-    TailRound R = tail_plan<NARROW>(A.kD, A.D, A.use_min, A.gpo, A.lpo, st, seg_global_min(first, nseg));
-    int err = 0;
-    while (!R.done) {
-        if (R.i > A.max_rounds) {
-            err = DUPIN_ERR_NO_PROGRESS;
-            break;
-        }
-        const long long i = R.i;
-        const long long *cur = segbuf + (i & 1) * nseg;  // minima at the start of round i
-        long long *nxt = segbuf + ((i + 1) & 1) * nseg;  // minima after round i
-        TailAcc<TAIL_WARPS> &acc = s_acc[i & 1];
-        // ---- select: lanes test segments in parallel; a candidate segment
-        // is then scanned by its warp (two vertices per lane)
-        unsigned long long wlo = 0, whi = 0;
-        long long mins = kMaxLL;  // new minimum over the segments this lane looked at
-        for (int q0 = wid * 32; q0 < nseg; q0 += TAIL_THREADS) {
-            const int q = q0 + lane;
-            const long long sm = q < nseg ? cur[q] : kMaxLL;
-            if (q < nseg) nxt[q] = sm;
-            const bool cand = seg_candidate(sm, R);
-            if (!cand) mins = sm < mins ? sm : mins;  // untouched by the select
-            unsigned cm = __ballot_sync(0xffffffffu, cand);
-            __syncwarp();
-            while (cm) {
-                const int qq = q0 + __ffs(cm) - 1;
-                cm &= cm - 1;
-                const long long p = (long long)qq * TAIL_SEG + 2 * lane;
-                const longlong2 v = *(const longlong2 *)&tw[p];
-                bool s0, s1;
-                if (R.minrule) {
-                    s0 = v.x >= 0 && v.x <= R.minw;
-                    s1 = v.y >= 0 && v.y <= R.minw;
-                } else {
-                    s0 = v.x >= 0 && (v.x <= R.gle || mul_le(v.x, R.Y, R.Xhi, R.Xlo));
-                    s1 = v.y >= 0 && (v.y <= R.gle || mul_le(v.y, R.Y, R.Xhi, R.Xlo));
-                }
-                long long m = kMaxLL;  // the segment's minimum over its survivors
-                if (v.x >= 0 && !s0) m = v.x;
-                if (v.y >= 0 && !s1 && v.y < m) m = v.y;
-                m = warp_min64(m);
-                if (lane == 0) {
-                    nxt[qq] = m;
-                    mins = m < mins ? m : mins;
-                }
-                const unsigned b0 = __ballot_sync(0xffffffffu, s0), b1 = __ballot_sync(0xffffffffu, s1);
-                if (b0 | b1) {
-                    unsigned base = 0;
-                    if (lane == 0) base = atomicAdd(&acc.F, (unsigned)(__popc(b0) + __popc(b1)));
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    const unsigned lt = (1u << lane) - 1u;
-                    unsigned slot = base + __popc(b0 & lt) + __popc(b1 & lt);
-                    if (s0) {
-                        tw[p] = -i;
-                        if (NARROW) wlo += (unsigned long long)v.x;
-                        else add128(wlo, whi, (unsigned long long)v.x, 0);
-                        tf[slot++] = (unsigned short)p;
-                    }
-                    if (s1) {
-                        tw[p + 1] = -i;
-                        if (NARROW) wlo += (unsigned long long)v.y;
-                        else add128(wlo, whi, (unsigned long long)v.y, 0);
-                        tf[slot] = (unsigned short)(p + 1);
-                    }
-                }
-            }
-        }
-        // the select's sums and minimum stay in registers: they are reduced
-        // with the expand's after it, off the path to the first barrier
-        __syncthreads();
-        // round i+1's counter was last read in round i-1: reset it now
-        if (tid == 0) s_acc[(i + 1) & 1].F = 0;
-        const int F = (int)acc.F;
-        // ---- expand
-        unsigned long long ilo = 0, ihi = 0;
-        long long mind = kMaxLL;
-        auto apply = [&](int v, long long c) {
-            const long long wv = tw[v];
-            if (wv >= 0) {
-                const long long old = (long long)atomicAdd((unsigned long long *)&tw[v], (unsigned long long)(-c));
-                atomicMin(&nxt[v / TAIL_SEG], old - c);
-                mind = old - c < mind ? old - c : mind;
-            } else if (wv == -i) {
-                if (NARROW) ilo += (unsigned long long)c;
-                else add128(ilo, ihi, (unsigned long long)c, 0);
-            }
-        };
-        // TAIL_ILP arcs per thread at a time: their loads from L2 are issued
-        // together before any of them is applied
-        auto arcs = [&](const long long (&pos)[TAIL_ILP]) {
-            int cv[TAIL_ILP];
-            long long cc[TAIL_ILP];
-#pragma unroll
-            for (int u = 0; u < TAIL_ILP; u++) {
-                if (pos[u] >= 0) {
-                    cv[u] = tcol[pos[u]];
-                    cc[u] = dg ? DUPIN_Q_ONE : tcw[pos[u]];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < TAIL_ILP; u++)
-                if (pos[u] >= 0) apply(cv[u], cc[u]);
-        };
-        if (F <= TAIL_FAST) {
-            // the frontier's arcs in chunks of 32 consecutive arcs of one
-            // vertex: chunk c goes to warp c % TAIL_WARPS, TAIL_ILP of a warp's
-            // chunks in flight at once; the walk is the same in every lane
-            // (broadcast shared loads, no divergence)
-            int e = 0, cbase = 0;
-            int p0 = F > 0 ? tf[0] : 0;
-            int a0 = F > 0 ? toff[p0] : 0, a1 = F > 0 ? toff[p0 + 1] : 0;
-            int c = wid;
-            while (e < F) {
-                long long pos[TAIL_ILP];
-                int got = 0;
-#pragma unroll
-                for (int u = 0; u < TAIL_ILP; u++) {
-                    pos[u] = -1;
-                    while (e < F && c >= cbase + ((a1 - a0 + 31) >> 5)) {
-                        cbase += (a1 - a0 + 31) >> 5;
-                        e++;
-                        if (e < F) {
-                            p0 = tf[e];
-                            a0 = toff[p0];
-                            a1 = toff[p0 + 1];
-                        }
-                    }
-                    if (e < F) {
-                        const int a = a0 + (c - cbase) * 32 + lane;
-                        if (a < a1) pos[u] = a;
-                        c += TAIL_WARPS;
-                        got++;
-                    }
-                }
-                if (got == 1) {  // one chunk: no predicated-off slots to issue
-                    if (pos[0] >= 0) apply(tcol[pos[0]], dg ? DUPIN_Q_ONE : tcw[pos[0]]);
-                } else {
-                    arcs(pos);
-                }
-            }
-        } else {
-            for (int c0 = 0; c0 < F; c0 += TAIL_THREADS) {
-                const int qq = c0 + tid;
-                long long deg = 0;
-                if (qq < F) {
-                    const int p = tf[qq];
-                    deg = toff[p + 1] - toff[p];
-                }
-                long long tot;
-                long long ex = block_excl_scan<TAIL_WARPS>(deg, s_w, tot);
-                s_pref[tid] = ex;
-                const int nq = (F - c0) < TAIL_THREADS ? (F - c0) : TAIL_THREADS;
-                if (tid == 0) s_pref[nq] = tot;
-                __syncthreads();
-                for (long long x0 = tid; x0 < tot; x0 += TAIL_ILP * TAIL_THREADS) {
-                    long long pos[TAIL_ILP];
-#pragma unroll
-                    for (int u = 0; u < TAIL_ILP; u++) {
-                        const long long x = x0 + (long long)u * TAIL_THREADS;
-                        pos[u] = -1;
-                        if (x < tot) {
-                            const int e = smem_last_le(s_pref, nq, x);
-                            const int p = tf[c0 + e];
-                            pos[u] = toff[p] + (x - s_pref[e]);
-                        }
-                    }
-                    arcs(pos);
-                }
-                __syncthreads();
-            }
-        }
-        if (NARROW) {
-            if (__any_sync(0xffffffffu, wlo != 0)) wlo = warp_sum64_redux(wlo);
-            if (__any_sync(0xffffffffu, ilo != 0)) ilo = warp_sum64_redux(ilo);
-        } else {
-            if (__any_sync(0xffffffffu, (wlo | whi) != 0)) warp_sum128(wlo, whi);
-            if (__any_sync(0xffffffffu, (ilo | ihi) != 0)) warp_sum128(ilo, ihi);
-        }
-        mins = warp_min64(mind < mins ? mind : mins);
-        if (lane == 0) {
-            acc.wlo[wid] = wlo;
-            acc.whi[wid] = whi;
-            acc.ilo[wid] = ilo;
-            acc.ihi[wid] = ihi;
-            acc.mins[wid] = mins;
-        }
-        __syncthreads();
-        // ---- every warp: close round i and plan round i + 1 (same values everywhere)
-        u128 wsel, internal;
-        long long mins_all;
-        tail_acc_sum<TAIL_WARPS, NARROW>(acc, wsel, internal, mins_all);
-        st.f = st.f - (wsel - (internal >> 1));
-        st.scan += L;
-        st.size -= F;
-        st.round = i;
-        st.n_min_rule += R.minrule ? 1 : 0;
-        // the best prefix and the trace are kept by the last warp alone: its
-        // select covers the fewest segments (the tail has at most 234 of 64)
-        if (wid == TAIL_WARPS - 1 && st.size > 0 && frac_gt<NARROW>(st.f, st.size, st.bf, st.best_size)) {
-            st.bf = st.f;
-            st.best_size = st.size;
-            st.best_round = i;
-        }
-        if (tid == (TAIL_WARPS - 1) * 32 && i < A.tr_cap) {
-            A.tr_f_hi[i] = (long long)(unsigned long long)(st.f >> 64);
-            A.tr_f_lo[i] = (unsigned long long)st.f;
-            A.tr_size[i] = st.size;
-            A.tr_peeled[i] = F;
-        }
-        if (F == 0) {  // cannot happen (Lemma 4.2 / minimum rule); stop instead of spinning
-            err = DUPIN_ERR_NO_PROGRESS;
-            break;
-        }
-        R = tail_plan<NARROW>(A.kD, A.D, A.use_min, A.gpo, A.lpo, st, mins_all);
-    }
-    if (tid == (TAIL_WARPS - 1) * 32) {
-        s_pref[0] = st.best_round;
-        s_pref[1] = st.best_size;
-        s_pref[2] = (long long)(unsigned long long)st.bf;
-        s_pref[3] = (long long)(unsigned long long)(st.bf >> 64);
-    }
+    const int err = local_rounds<TAIL_THREADS, NARROW>(S, G, st, s_acc, s_rows, s_hand);
     __syncthreads();
     for (long long p = tid; p < L; p += TAIL_THREADS) {
-        const long long wv = tw[p];
+        const long long wv = S.tw[p];
         if (wv < 0) A.pr[live[p]] = (int)(-wv);
     }
-    if (tid == 0) {
-        st.best_round = s_pref[0];
-        st.best_size = s_pref[1];
-        st.bf = mk128((unsigned long long)s_pref[2], (unsigned long long)s_pref[3]);
+    if (tid == (TAIL_WARPS - 1) * 32) {
         if (err) set_error(ctl, err);
         ctl->round = st.round;
         ctl->size = st.size;
@@ -1351,15 +1119,15 @@ __device__ __forceinline__ void peel_tail_body(const PeelArgs &A, unsigned char 
 __global__ void __launch_bounds__(TAIL_THREADS, 1) k_peel_tail(PeelArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TailAcc<TAIL_WARPS> s_acc[2];
-    __shared__ long long s_w[TAIL_WARPS];
-    __shared__ long long s_pref[TAIL_THREADS + 1];
+    __shared__ unsigned s_rows[64 * TAIL_WARPS];
+    __shared__ LocalHand s_hand;
     const PeelCtl *ctl = A.ctl;
     if (ctl->status != ST_TAIL || ctl->error) return;
     // f only decreases, and a round's sums (removed weights, arcs inside
     // the removed set) are at most 2f; the best f so far must fit 64 bits too
     if (ctl->f_hi == 0 && ctl->f_lo < (1ull << 62) && ctl->bf_hi == 0)
-        peel_tail_body<true>(A, smem, s_acc, s_w, s_pref);
-    else peel_tail_body<false>(A, smem, s_acc, s_w, s_pref);
+        peel_tail_body<true>(A, smem, s_acc, s_rows, &s_hand);
+    else peel_tail_body<false>(A, smem, s_acc, s_rows, &s_hand);
 }
 
 // best_mask[u] = (peel_round[u] > best_round) for a best round known on the host
@@ -1411,29 +1179,28 @@ int peel_grid_size() {
 }
 
 // raise k_peel_tail's dynamic shared-memory limit, once per device (the
-// limit is a per-device attribute of the function)
-static int set_tail_smem() {
+// limit is a per-device attribute of the function); every launch takes all of
+// it, for the sub-graph's arcs beside the vertex state
+static int set_tail_smem(int *bytes) {
     static std::mutex mu;
-    static bool done[64] = {false};
+    static int done[64] = {0};
     int dev = 0, smem = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return dupin_fail(DUPIN_ERR_CUDA, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(mu);
+    *bytes = done[dev];
     if (done[dev]) return DUPIN_OK;
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, k_peel_tail);
     if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncGetAttributes(k_peel_tail)");
+    if (local_bytes(tail_cap_limit(), 4) > smem - (int)fa.sharedSizeBytes)
+        return dupin_fail(DUPIN_ERR_CUDA, "the one-CTA tail's state does not fit its shared memory");
     int dyn = smem - (int)fa.sharedSizeBytes;
     e = cudaFuncSetAttribute(k_peel_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncSetAttribute(k_peel_tail)");
-    done[dev] = true;
+    *bytes = done[dev] = dyn;
     return DUPIN_OK;
-}
-
-static long long tail_smem_bytes(long long cap) {
-    const long long nseg = (cap + TAIL_SEG - 1) / TAIL_SEG;
-    return 8 * nseg * TAIL_SEG + 16 * nseg + 4 * (cap + 1) + 2 * cap + 16;
 }
 
 static int check_params(const dupin_graph *g, const dupin_params *p) {
@@ -1696,12 +1463,8 @@ static PeelArgs make_args(const dupin_graph *g, const PeelWorkspace *ws, const d
     A.cl_c = plan.cl_cap > 0 ? cluster_ctas() : 0;
     A.dmat = ws->tbuf;
     A.again = 0;
-    {  // the dense tail's element: the weights without their common low zero bits
-        const unsigned long long o = p->metric == DUPIN_DG ? (unsigned long long)DUPIN_Q_ONE : g->w_or;
-        A.dshift = o ? __builtin_ctzll(o) : 0;
-        A.desz = (o >> A.dshift) >> 32 ? 8 : ((o >> A.dshift) >> 8 ? 4 : 1);
-        if (A.desz == 8) A.dshift = 0;
-    }
+    A.tail_smem = 0;
+    dense_element(p->metric == DUPIN_DG ? (unsigned long long)DUPIN_Q_ONE : g->w_or, &A.desz, &A.dshift);
     // (without the minimum rule a peel has few rounds, and the dense tail's
     // launches would cost more than it gains)
     A.dcap = plan.cl_cap > 0 && A.use_min && g->arcs > DUPIN_ONE_CTA_ARCS
@@ -1797,8 +1560,10 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
     auto tails = [&]() -> int {
         int rc2;
         if (plan.tail_cap > 0) {
-            if ((rc2 = set_tail_smem())) return rc2;
-            k_peel_tail<<<1, TAIL_THREADS, (size_t)tail_smem_bytes(plan.tail_cap), s>>>(A);
+            int dyn = 0;
+            if ((rc2 = set_tail_smem(&dyn))) return rc2;
+            A.tail_smem = dyn;
+            k_peel_tail<<<1, TAIL_THREADS, (size_t)dyn, s>>>(A);
         }
         if (plan.cl_cap > 0 && (rc2 = launch_cluster_tail(A, s))) return rc2;
         if (A.dcap > 0) {  // from the grid-wide rounds, or after the cluster tail
@@ -1943,9 +1708,12 @@ int launch_small_graph_peel(const PeelArgs &A, int metric, bool check, cudaStrea
     int rc = launch_init_weights(A.g, metric, A.w, A.pr, A.live0, A.ctl, check, s);
     if (rc) return rc;
     k_init_finish<<<1, 1, 0, s>>>(A, A.g.n);
-    rc = set_tail_smem();
+    PeelArgs B = A;
+    int dyn = 0;
+    rc = set_tail_smem(&dyn);
     if (rc) return rc;
-    k_peel_tail<<<1, TAIL_THREADS, (size_t)tail_smem_bytes(A.tail_cap), s>>>(A);
+    B.tail_smem = dyn;
+    k_peel_tail<<<1, TAIL_THREADS, (size_t)dyn, s>>>(B);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return dupin_cuda_fail(e, "small-graph peel kernels");
     return DUPIN_OK;
