@@ -739,6 +739,7 @@ __device__ __forceinline__ void cluster_body(const PeelArgs &A, const int P, uns
         const long long wv = s < nown ? tw[s] : -1;
         const int u = s < nown ? live[s * C + r] : 0;
         if (s < nown && wv < 0) A.pr[u] = (int)(-wv);
+        if (hand != ST_DONE && s < nown && wv < 0) atomicAnd(&A.rank[u >> 5].live, ~(1u << (u & 31)));
         if (hand != ST_DONE) {
             const unsigned bal = __ballot_sync(0xffffffffu, wv >= 0);
             int base = 0;

@@ -621,8 +621,7 @@ __global__ void k_dense_clear(PeelArgs A) {
 // The live arcs of every live vertex's row, written into the matrix: one walk
 // over the rows (the sparse tails' builds need two: a count and a fill).
 __global__ void __launch_bounds__(BULK_THREADS) k_dense_fill(PeelArgs A) {
-    __shared__ long long s_base[WALK_WIN + 1];
-    __shared__ long long s_start[WALK_WIN + 1];
+    __shared__ WalkShared s_walk;
     __shared__ long long s_k0;
     __shared__ unsigned s_cnt;
     const PeelCtl *c = A.ctl;
@@ -647,20 +646,34 @@ __global__ void __launch_bounds__(BULK_THREADS) k_dense_fill(PeelArgs A) {
     const int *col = A.g.col;
     const int *hubs = A.g.hubs;
     const long long *cw = A.g.cw;
-    const int *pr = A.pr;
+    const RankWord *rank = A.rank;
     const size_t pitch = (size_t)A.cl_c * dense_slice(L, A.cl_c);
     unsigned cnt = 0;
-    walk_arcs([=](long long k) { return tdeg[k]; }, [=](long long k) { return rp[live[k]]; }, L, e0, e1, k0, s_base,
-              s_start, [&](long long k, long long pos) {
-                  const int v = arc_head(col[pos], hubs);
-                  if (pr[v] != DUPIN_LIVE) return;
-                  const size_t at = (size_t)k * pitch + (size_t)A.loc[v];
-                  const unsigned long long q = (unsigned long long)(cw ? cw[pos] : DUPIN_Q_ONE) >> A.dshift;
-                  if (A.desz == 1) ((unsigned char *)A.dmat)[at] = (unsigned char)q;
-                  else if (A.desz == 4) ((unsigned *)A.dmat)[at] = (unsigned)q;
-                  else ((long long *)A.dmat)[at] = (long long)q;
-                  cnt++;
-              });
+    walk_arcs<BULK_THREADS, BUILD_ILP, true>(
+        [=](long long k) { return tdeg[k]; }, [=](long long k) { return rp[live[k]]; }, L, e0, e1, k0, s_walk,
+        [&](const long long (&k)[BUILD_ILP], const long long (&pos)[BUILD_ILP]) {
+            int v[BUILD_ILP], to[BUILD_ILP];
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) v[u] = pos[u] >= 0 ? col[pos[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) {
+                if (v[u] < 0) v[u] = hubs[-v[u] - 1];
+                if (pos[u] >= 0 && !((rank[v[u] >> 5].live >> (v[u] & 31)) & 1u)) v[u] = -1;
+                if (pos[u] < 0) v[u] = -1;
+            }
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) to[u] = v[u] >= 0 ? A.loc[v[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) {
+                if (v[u] < 0) continue;
+                const size_t at = (size_t)k[u] * pitch + (size_t)to[u];
+                const unsigned long long q = (unsigned long long)(cw ? cw[pos[u]] : DUPIN_Q_ONE) >> A.dshift;
+                if (A.desz == 1) ((unsigned char *)A.dmat)[at] = (unsigned char)q;
+                else if (A.desz == 4) ((unsigned *)A.dmat)[at] = (unsigned)q;
+                else ((long long *)A.dmat)[at] = (long long)q;
+                cnt++;
+            }
+        });
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if ((threadIdx.x & 31) == 0) atomicAdd(&s_cnt, cnt);
     __syncthreads();

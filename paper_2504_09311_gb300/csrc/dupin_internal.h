@@ -29,11 +29,11 @@ struct PeelWorkspace {
     long long n = 0, arcs = 0, tail_cap = 0, tr_cap = 0, tarc_cap = 0;
     int grid = 0;    // blocks of the persistent kernel
     int device = 0;  // where it was allocated
-    long long *w = nullptr;
+    long long *w = nullptr, *w2 = nullptr;
     int *pr = nullptr;
     int *live0 = nullptr, *live1 = nullptr;
-    int *stage_id = nullptr;
-    long long *stage_start = nullptr, *stage_off = nullptr;
+    long long *stage_start = nullptr;
+    int *stage_deg = nullptr;
     long long *fstart = nullptr, *fbase = nullptr;
     long long *cstart = nullptr;
     BlockPart *part = nullptr;
@@ -50,6 +50,7 @@ struct PeelWorkspace {
     uint8_t *tbuf = nullptr;  // holds tcw and tcol, or the dense tail's matrix
     long long tbuf_bytes = 0;
     uint8_t *mask = nullptr;
+    RankWord *rank = nullptr;
     bool async = false;  // allocated with cudaMallocAsync (freed with cudaFreeAsync)
     // DUPIN_TIMING: init start, init done, grid-wide rounds start and done,
     // build start and done, tail done
@@ -128,7 +129,7 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
 int peel_finish(const dupin_graph *g, PeelWorkspace *ws, const dupin_params *p, dupin_result *r, cudaStream_t s);
 
 // kernels shared by loading and peeling
-int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, int *live0, PeelCtl *ctl,
+int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, int *live0, RankWord *rank, PeelCtl *ctl,
                         bool check, cudaStream_t s);
 
 // batched one-CTA-per-graph peels (batch.cu)

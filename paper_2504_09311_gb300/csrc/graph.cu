@@ -359,7 +359,7 @@ extern "C" int dupin_graph_load(const dupin_graph_desc *d, void *stream, dupin_g
         dg.a = g->a;
         dg.key = fingerprint_key();
         rc = DUPIN_OK;
-        if (e == cudaSuccess && dg.cw) rc = launch_init_weights(dg, DUPIN_DW, w, nullptr, nullptr, ctl, true, s);
+        if (e == cudaSuccess && dg.cw) rc = launch_init_weights(dg, DUPIN_DW, w, nullptr, nullptr, nullptr, ctl, true, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctl, sizeof(PeelCtl), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         gfree(w, s);

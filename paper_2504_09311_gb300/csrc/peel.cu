@@ -46,7 +46,7 @@
 // ------------------------------------------------------------- (a) init
 
 // w_u = a_u (DW/FD) or deg_u * 1.0 (DG); every vertex live; live list = ids.
-__global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *live0, PeelCtl *ctl) {
+__global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *live0, RankWord *rank, PeelCtl *ctl) {
     long long n = g.n;
     unsigned long long lo = 0, hi = 0;
     long long mn = kMaxLL;
@@ -63,6 +63,7 @@ __global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *li
         w[u] = wu;
         if (pr) pr[u] = DUPIN_LIVE;
         if (live0) live0[u] = (int)u;
+        if (rank && (u & 31) == 0) rank[u >> 5] = RankWord{~0u, ~0u, (unsigned)u, 0};  // bits past n are never asked for
     }
     if (dg) {
         warp_sum128(lo, hi);
@@ -271,6 +272,142 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
     }
 }
 
+// The same sums without the checks, for peeling: tiles of IT_TILE arc weights
+// arrive in shared memory by bulk copies, two buffers per block; a block scan
+// turns a tile into its running sums (a thread takes eight neighbours, reading
+// its four 16-byte pieces in an order that spreads a quarter-warp over the
+// banks), and each row inside the tile is the difference of two of them: a
+// store per row, in row order.  Rows that cross a tile's edge are added up with
+// atomics (w holds a_u from k_init_vertex).  Sums wrap like any 64-bit ones.
+// The arc-balanced form above finds each arc's row by shuffles and scans rows
+// in registers: issue-bound, 1.76 ms on R-MAT scale 24 (4.2 GB of weights).
+#define IT_THREADS 256
+#define IT_ITEMS 8
+#define IT_TILE (IT_THREADS * IT_ITEMS)
+
+__device__ __forceinline__ void it_load(long long *buf, const long long *src, unsigned bytes, unsigned long long *mb) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(buf), m = (unsigned)__cvta_generic_to_shared(mb);
+    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(m), "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d), "l"(src),
+                 "r"(bytes), "r"(m)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long *w, PeelCtl *ctl) {
+    __shared__ __align__(128) long long s_buf[2][IT_TILE];
+    __shared__ unsigned long long s_mb[2];
+    __shared__ long long s_w[IT_THREADS / 32], s_row;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const long long A = g.arcs, n = g.n;
+    const long long tiles = (A + IT_TILE - 1) / IT_TILE;
+    const long long T0 = split_at(tiles, blockIdx.x, gridDim.x), T1 = split_at(tiles, blockIdx.x + 1, gridDim.x);
+    if (T0 >= T1) return;
+    if (tid < 2)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&s_mb[tid])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    __syncthreads();
+    auto bytes_of = [&](long long t) {
+        const long long left = A - t * IT_TILE;
+        return (unsigned)(8 * (left < IT_TILE ? left : IT_TILE));  // an even number of arcs: a multiple of 16
+    };
+    if (tid == 0)
+        for (int k = 0; k < 2 && T0 + k < T1; k++) it_load(s_buf[k], g.cw + (T0 + k) * IT_TILE, bytes_of(T0 + k), &s_mb[k]);
+    if (tid < 32) {
+        const long long r = warp_search_last_le(g.rp, n, T0 * IT_TILE);  // the row of the first arc (the last of equal starts)
+        if (lane == 0) s_row = r;
+    }
+    __syncthreads();
+    long long r0 = s_row;
+    for (long long t = T0; t < T1; t++) {
+        const int k = (int)((t - T0) & 1);
+        const unsigned parity = (unsigned)(((t - T0) >> 1) & 1);
+        long long *P = s_buf[k];
+        const long long t0 = t * IT_TILE;
+        const int len = (int)(A - t0 < IT_TILE ? A - t0 : IT_TILE);
+        bool bad = false;
+        {
+            const unsigned m = (unsigned)__cvta_generic_to_shared(&s_mb[k]);
+            unsigned done = 0;
+            for (long long it = 0; !done; it++) {
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, "
+                    "p;\n\t}"
+                    : "=r"(done)
+                    : "r"(m), "r"(parity)
+                    : "memory");
+                if (!done && it > DUPIN_SPIN_LIMIT) {  // a lost copy: cannot happen; give up rather than hang
+                    bad = true;
+                    break;
+                }
+            }
+        }
+        if (__syncthreads_or(bad)) {
+            if (tid == 0) set_error(ctl, DUPIN_ERR_TIMEOUT);
+            return;
+        }
+        // this thread's eight arcs: piece c at arcs 8 tid + 2 c
+        longlong2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = (q + (tid >> 1)) & 3;
+            const longlong2 x = *(const longlong2 *)&P[IT_ITEMS * tid + 2 * c];
+#pragma unroll
+            for (int z = 0; z < 4; z++)
+                if (c == z) v[z] = x;
+        }
+        long long sum = 0;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            const int at = IT_ITEMS * tid + 2 * c;
+            const long long x = at < len ? v[c].x : 0, y = at < len ? v[c].y : 0;  // len is even
+            v[c].x = sum;
+            v[c].y = sum + x;
+            sum += x + y;
+        }
+        long long total;
+        const long long before = block_excl_scan<IT_THREADS / 32>(sum, s_w, total);  // ends with a barrier
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = (q + (tid >> 1)) & 3;
+            longlong2 x;
+#pragma unroll
+            for (int z = 0; z < 4; z++)
+                if (c == z) x = v[z];
+            x.x += before;
+            x.y += before;
+            *(longlong2 *)&P[IT_ITEMS * tid + 2 * c] = x;
+        }
+        __syncthreads();
+        // rows that start before the tile's end, from the one holding its first arc on
+        const long long t1 = t0 + len;
+        for (long long rb = r0;; rb += IT_THREADS) {
+            const long long r = rb + tid;
+            long long b = t1, e = t1;
+            if (r < n) {
+                b = g.rp[r];
+                e = g.rp[r + 1];
+            }
+            if (b < t1) {
+                const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
+                if (hi > lo) {
+                    const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
+                    if (b >= t0 && e <= t1) w[r] = s + (g.a ? g.a[r] : 0);
+                    else atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
+                }
+                if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
+            }
+            if (__syncthreads_or(r >= n || b >= t1)) break;
+        }
+        r0 = s_row;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // reads and writes of P before the next copy into it
+        __syncthreads();
+        if (tid == 0 && t + 2 < T1) {
+            it_load(P, g.cw + (t + 2) * IT_TILE, bytes_of(t + 2), &s_mb[k]);
+        }
+    }
+}
+
 // sum over u of (w_u + a_u) and min w (DW/FD)
 __global__ void k_init_reduce(DevGraph g, const long long *w, PeelCtl *ctl) {
     unsigned long long lo = 0, hi = 0;
@@ -294,19 +431,19 @@ __global__ void k_init_reduce(DevGraph g, const long long *w, PeelCtl *ctl) {
     }
 }
 
-int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, int *live0, PeelCtl *ctl, bool check,
-                        cudaStream_t s) {
+int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, int *live0, RankWord *rank, PeelCtl *ctl,
+                        bool check, cudaStream_t s) {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int vgrid = sms * 8;
     const bool isdg = metric == DUPIN_DG || dg.cw == nullptr;
-    k_init_vertex<<<vgrid, 256, 0, s>>>(dg, isdg ? 1 : 0, w, pr, live0, ctl);
+    k_init_vertex<<<vgrid, 256, 0, s>>>(dg, isdg ? 1 : 0, w, pr, live0, rank, ctl);
     if (!isdg) {
         if (dg.arcs > 0) {
             int agrid = sms * 8;
             if (check) k_init_arcs<true><<<agrid, INIT_THREADS, 0, s>>>(dg, w, ctl);
-            else k_init_arcs<false><<<agrid, INIT_THREADS, 0, s>>>(dg, w, ctl);
+            else k_init_tiles<<<(int)std::min<long long>(sms * 6, (dg.arcs + IT_TILE - 1) / IT_TILE), IT_THREADS, 0, s>>>(dg, w, ctl);
         }
         k_init_reduce<<<vgrid, 256, 0, s>>>(dg, w, ctl);
     }
@@ -371,7 +508,22 @@ __device__ __forceinline__ void stage_entry(const PeelArgs &A, long long j0, boo
     if (stage) {
         const long long slot = (long long)base + __popc(bal & ((1u << lane) - 1u));
         A.stage_start[j0 + slot] = start;
-        A.stage_off[j0 + slot] = deg;
+        A.stage_deg[j0 + slot] = (int)deg;
+    }
+}
+
+// The lanes with 'gone' set take vertex id's bit out of the live bits, one
+// atomic per word and warp (in round 1 a warp's 32 vertices share one or two
+// words).
+__device__ __forceinline__ void clear_live(RankWord *rank, int id, bool gone) {
+    unsigned left = __ballot_sync(0xffffffffu, gone);
+    while (left) {
+        const int word = __shfl_sync(0xffffffffu, id >> 5, __ffs(left) - 1);
+        const bool mine = gone && (id >> 5) == word;
+        const unsigned bits = __reduce_or_sync(0xffffffffu, mine ? 1u << (id & 31) : 0u);
+        const unsigned same = __ballot_sync(0xffffffffu, mine);
+        if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAnd(&rank[word].live, ~bits);
+        left &= ~same;
     }
 }
 
@@ -384,8 +536,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
     __shared__ unsigned s_nst;   // frontier entries staged by the block
     __shared__ unsigned s_surv;  // candidates / survivors placed by the block
     __shared__ long long s_scan[BULK_WARPS];
-    __shared__ long long s_base[WALK_WIN + 1];
-    __shared__ long long s_start[WALK_WIN + 1];
+    __shared__ WalkShared s_walk;
     __shared__ int s_hub[DUPIN_HUB_MAX];
     // a round's decrements of each hub, as two 32-bit words (hi gets the carries)
     __shared__ unsigned s_hlo[DUPIN_HUB_MAX], s_hhi[DUPIN_HUB_MAX];
@@ -394,6 +545,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
     // block barrier publishes it.  s_rd carries phase B's totals to phase D.
     __shared__ RoundState s_st;
     __shared__ long long s_elive;  // |E(S)|
+    __shared__ int s_moved;        // the live list was compacted: weights stand by position
     __shared__ struct {
         unsigned long long wlo, whi;  // sum of the selected vertices' weights
         long long U_sel, newSize;
@@ -431,11 +583,32 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         st.n_min_rule = ctl->n_min_rule;
         st.scan = ctl->scan_volume;
         s_elive = ctl->elive;
+        s_moved = 0;
         s_rd.U_sel = kMaxLL;  // no round yet
         s_rd.arcs = kMaxLL;
     }
     __syncthreads();
     if (ctl->status != ST_RUNNING || ctl->error) return;
+    if (ctl->handed) {
+        // given back by a cluster tail: every vertex listed again, the dead ones
+        // as gone (the live bits and the weights by id are up to date)
+        const long long nw = (g.n + 31) >> 5;
+        for (long long q = split_at(nw, b, G) + wid; q < split_at(nw, b + 1, G); q += BULK_WARPS) {
+            const unsigned lv = A.rank[q].live;
+            const long long u = 32 * q + lane;
+            if (u < g.n) A.live0[u] = (lv >> lane) & 1u ? (int)u : -1;
+            if (lane == 0) {
+                A.rank[q].listed = ~0u;
+                A.rank[q].first = (unsigned)(32 * q);
+            }
+        }
+        if (!grid_barrier(ctl, G, bar_target)) return;
+        if (tid == 0) {
+            s_st.live_sel = 0;
+            s_st.live_len = g.n;
+        }
+        __syncthreads();
+    }
 
     for (;;) {
         const long long size = s_st.size;
@@ -444,7 +617,8 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         // vertices or arcs costs a tail microseconds and the grid-wide kernel
         // its barriers)
         const bool small_round = s_rd.U_sel <= DUPIN_TAIL_SMALL_ROUND || s_rd.arcs <= DUPIN_TAIL_SMALL_ARCS;
-        if (size == 0 || (size <= A.hcap && (2 * s_elive <= A.tail_arcs || (small_round && 2 * s_elive <= A.tarc_cap))))
+        // (and the live list holds nobody else)
+        if (size == 0 || (size <= A.hcap && s_st.live_len == size && (2 * s_elive <= A.tail_arcs || (small_round && 2 * s_elive <= A.tarc_cap))))
             break;
         if (s_st.round >= A.max_rounds) {
             if (b == 0 && tid == 0) set_error(ctl, DUPIN_ERR_NO_PROGRESS);
@@ -483,6 +657,8 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         const int live_sel = s_st.live_sel;
         int *live = live_sel ? A.live1 : A.live0;
         int *nlive = live_sel ? A.live0 : A.live1;
+        long long *wl = live_sel ? A.w2 : A.w;   // the listed vertices' weights ...
+        long long *nwl = live_sel ? A.w : A.w2;  // ... and where a compaction moves them
         const long long L = s_st.live_len;
         const long long j0 = split_at(L, b, G), j1 = split_at(L, b + 1, G);
         // Phase A selects w <= T.  When k(1+eps) < 2 the threshold can select
@@ -504,7 +680,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
                 const long long j = jb + lane;
                 int id = j < j1 ? live[j] : -1;
                 long long wv = 0;
-                if (id >= 0) wv = A.w[id];
+                if (id >= 0) wv = wl[j];
                 const bool sel = id >= 0 && wv <= thr;
                 if (id >= 0 && !sel) {
                     surv++;
@@ -520,6 +696,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
                     deg = g.rp[id + 1] - start;
                     sdeg += deg;
                 }
+                clear_live(A.rank, id, sel);
                 stage_entry(A, j0, sel && deg > 0, start, deg, &s_nst);
             }
             BlockRed<BULK_WARPS, 6> r;
@@ -550,7 +727,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
                 for (long long jb = j0 + wid * 32; jb < j1; jb += BULK_THREADS) {
                     const long long j = jb + lane;
                     const int id = j < j1 ? live[j] : -1;
-                    const long long wv = id >= 0 ? A.w[id] : kMaxLL;
+                    const long long wv = id >= 0 ? wl[j] : kMaxLL;
                     const bool c = id >= 0 && wv == m;
                     if (id >= 0 && wv > m && wv < min2) min2 = wv;
                     const unsigned cb = __ballot_sync(0xffffffffu, c);
@@ -667,12 +844,15 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             for (long long c = tid; c < myCand; c += BULK_THREADS) {
                 const long long j = A.stage_id[j0 + c];
                 A.pr[live[j]] = (int)i;
+                atomicAnd(&A.rank[live[j] >> 5].live, ~(1u << (live[j] & 31)));
                 live[j] = -1;
             }
             __syncthreads();
         }
         const long long newSize = size - U_sel;
         const bool compact = newSize > 0 && (2 * newSize <= L || newSize <= A.hcap);
+        // a compaction reads the live bits of words that other blocks' candidates share
+        if (minrule && compact && !grid_barrier(ctl, G, bar_target)) return;
         if (tid == 0) {
             s_rd.U_sel = U_sel;
             s_rd.arcs = totArcs;
@@ -684,9 +864,9 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         // and starts its walk at the frontier entry holding its first arc.  The
         // consumers whose first arc lies in this block's entries, global arcs
         // [arcBase, arcBase + myDeg), are c_lo .. c_lo + nc - 1; their first
-        // arcs go to shared memory (s_base is free until phase C), and every
+        // arcs go to shared memory (the walk's window, free until phase C), and every
         // entry finds its consumers there by binary search.
-        long long *s_cs = s_base;
+        long long *s_cs = s_walk.off;
         long long c_lo = 0, nc = 0;
         if (myDeg > 0) {
             const unsigned long long T = (unsigned long long)totArcs;
@@ -701,7 +881,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         long long carry = 0;
         for (long long q0 = 0; q0 < myStage; q0 += BULK_THREADS) {
             const long long q = q0 + tid;
-            const long long deg = q < myStage ? A.stage_off[j0 + q] : 0;
+            const long long deg = q < myStage ? A.stage_deg[j0 + q] : 0;
             long long chunk;
             const long long off = carry + block_excl_scan<BULK_WARPS>(deg, s_scan, chunk);
             carry += chunk;
@@ -721,20 +901,33 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             }
         }
         if (b == 0 && tid == 0) A.fbase[U_stage] = totArcs;
-        if (compact) {
-            if (tid == 0) s_surv = 0;
-            __syncthreads();
-            for (long long jb = j0 + wid * 32; jb < j1; jb += BULK_THREADS) {
+        if (compact) {  // in id order: each warp a contiguous part of the slice
+            const long long c0 = j0 + split_at(j1 - j0, wid, BULK_WARPS), c1 = j0 + split_at(j1 - j0, wid + 1, BULK_WARPS);
+            long long kept = 0;
+            for (long long jb = c0; jb < c1; jb += 32) {
                 const long long j = jb + lane;
-                int id = j < j1 ? live[j] : -1;
-                const bool keep = id >= 0;
-                const unsigned bal = __ballot_sync(0xffffffffu, keep);
-                if (bal) {
-                    unsigned base = 0;
-                    if (lane == 0) base = atomicAdd(&s_surv, (unsigned)__popc(bal));
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    if (keep) nlive[survBase + (long long)base + __popc(bal & ((1u << lane) - 1u))] = id;
+                kept += __popc(__ballot_sync(0xffffffffu, j < c1 && live[j] >= 0));
+            }
+            if (lane == 0) s_scan[wid] = kept;
+            __syncthreads();
+            long long at = survBase;
+            for (int q = 0; q < wid; q++) at += s_scan[q];
+            for (long long jb = c0; jb < c1; jb += 32) {
+                const long long j = jb + lane;
+                const int id = j < c1 ? live[j] : -1;
+                const unsigned bal = __ballot_sync(0xffffffffu, id >= 0);
+                if (id >= 0) {
+                    const long long k = at + __popc(bal & ((1u << lane) - 1u));
+                    nlive[k] = id;
+                    nwl[k] = wl[j];
+                    RankWord *rw = &A.rank[id >> 5];
+                    const unsigned lv = rw->live;
+                    if ((lv & ((1u << (id & 31)) - 1u)) == 0) {  // the word's first live vertex
+                        rw->listed = lv;
+                        rw->first = (unsigned)k;
+                    }
                 }
+                at += __popc(bal);
             }
         }
         if (!grid_barrier(ctl, G, bar_target)) return;
@@ -754,72 +947,57 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             const int *col = g.col;
             const long long *cw = g.cw;
             int *pr = A.pr;
-            long long *w = A.w;
-            long long e = E0, kk = E0 < E1 ? A.cstart[b] : 0;
-            while (e < E1) {  // block-uniform
-                __syncthreads();
-                for (int t = tid; t <= WALK_WIN; t += BULK_THREADS) {
-                    const long long idx = kk + t;
-                    s_base[t] = idx <= U_stage ? fb[idx] : kMaxLL;
-                    s_start[t] = idx < U_stage ? fs[idx] : 0;
-                }
-                __syncthreads();
-                const long long wend = s_base[WALK_WIN];
-                const long long hi = E1 < wend ? E1 : wend;
-                for (long long xb = e + tid; xb < hi; xb += (long long)BULK_ILP * BULK_THREADS) {
-                    long long pos[BULK_ILP];
+            long long *w = compact ? nwl : wl;
+            if (E0 < E1) {
+                walk_arcs<BULK_THREADS, BULK_ILP, false>(
+                    [=](long long k) { return fb[k]; }, [=](long long k) { return fs[k]; }, U_stage, E0, E1, A.cstart[b], s_walk,
+                    [&](const long long (&)[BULK_ILP], const long long (&pos)[BULK_ILP]) {
+                        int cv[BULK_ILP], hv[BULK_ILP];
+                        long long cc[BULK_ILP];
 #pragma unroll
-                    for (int u = 0; u < BULK_ILP; u++) {
-                        const long long x = xb + (long long)u * BULK_THREADS;
-                        const int t = smem_last_le_fixed(s_base, x);
-                        pos[u] = x < hi ? s_start[t] + (x - s_base[t]) : -1;
-                    }
-                    int cv[BULK_ILP];
-                    long long cc[BULK_ILP];
-#pragma unroll
-                    for (int u = 0; u < BULK_ILP; u++) {
-                        if (pos[u] >= 0) {
-                            cv[u] = col[pos[u]];
-                            cc[u] = dg ? DUPIN_Q_ONE : cw[pos[u]];
-                        }
-                    }
-                    int pp[BULK_ILP];
-#pragma unroll
-                    for (int u = 0; u < BULK_ILP; u++)
-                        if (pos[u] >= 0) pp[u] = pr[cv[u] >= 0 ? cv[u] : s_hub[-cv[u] - 1]];
-#pragma unroll
-                    for (int u = 0; u < BULK_ILP; u++) {
-                        if (pos[u] < 0) continue;
-                        const int p = pp[u];
-                        const long long c = cc[u];
-                        if (p > (int)i) {
-                            const int cvu = cv[u];
-                            if (cvu >= 0) {
-                                if (A.lpo) {
-                                    const long long nv =
-                                        (long long)atomicAdd((unsigned long long *)&w[cvu], (unsigned long long)(-c)) - c;
-                                    mindec = nv < mindec ? nv : mindec;
-                                } else {
-                                    // result unused: a fire-and-forget reduction
-                                    atomicAdd((unsigned long long *)&w[cvu], (unsigned long long)(-c));
-                                }
-                            } else {  // hub head: aggregate in shared memory
-                                const int h = -cvu - 1;
-                                const unsigned cl = (unsigned)c;
-                                const unsigned old = atomicAdd(&s_hlo[h], cl);
-                                const unsigned ch =
-                                    (unsigned)((unsigned long long)c >> 32) + (old + cl < old ? 1u : 0u);
-                                if (ch) atomicAdd(&s_hhi[h], ch);
+                        for (int u = 0; u < BULK_ILP; u++) {
+                            cv[u] = 0;
+                            cc[u] = 0;
+                            if (pos[u] >= 0) {  // read once: kept out of the way of w and the rank words in L2
+                                cv[u] = __ldcs(col + pos[u]);
+                                cc[u] = dg ? DUPIN_Q_ONE : __ldcs(cw + pos[u]);
                             }
-                            nrem += 2;
-                        } else if (p == (int)i) {
-                            add128(ilo, ihi, (unsigned long long)c, 0);
-                            nrem++;
                         }
-                    }
-                }
-                kk += smem_last_le(s_base, WALK_WIN + 1, hi);
-                e = hi;
+                        RankWord rw[BULK_ILP];
+#pragma unroll
+                        for (int u = 0; u < BULK_ILP; u++) {
+                            hv[u] = cv[u] >= 0 ? cv[u] : s_hub[-cv[u] - 1];
+                            if (pos[u] >= 0) rw[u] = rank_word(A.rank, hv[u]);
+                        }
+#pragma unroll
+                        for (int u = 0; u < BULK_ILP; u++) {
+                            if (pos[u] < 0) continue;
+                            const long long c = cc[u];
+                            if (rank_live(rw[u], hv[u])) {
+                                const int cvu = cv[u];
+                                if (cvu >= 0) {
+                                    unsigned long long *to = (unsigned long long *)&w[rank_pos(rw[u], cvu)];
+                                    if (A.lpo) {
+                                        const long long nv = (long long)atomicAdd(to, (unsigned long long)(-c)) - c;
+                                        mindec = nv < mindec ? nv : mindec;
+                                    } else {
+                                        // result unused: a fire-and-forget reduction
+                                        atomicAdd(to, (unsigned long long)(-c));
+                                    }
+                                } else {  // hub head: aggregate in shared memory
+                                    const int h = -cvu - 1;
+                                    const unsigned cl = (unsigned)c;
+                                    const unsigned old = atomicAdd(&s_hlo[h], cl);
+                                    const unsigned ch = (unsigned)((unsigned long long)c >> 32) + (old + cl < old ? 1u : 0u);
+                                    if (ch) atomicAdd(&s_hhi[h], ch);
+                                }
+                                nrem += 2;
+                            } else if (pr[hv[u]] == (int)i) {
+                                add128(ilo, ihi, (unsigned long long)c, 0);
+                                nrem++;
+                            }
+                        }
+                    });
             }
         }
         if (nh > 0) {  // one reduction per hub touched by this block
@@ -827,8 +1005,9 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             for (int h = tid; h < nh; h += BULK_THREADS) {
                 const unsigned long long a = ((unsigned long long)s_hhi[h] << 32) + s_hlo[h];
                 if (a) {
-                    const long long nv =
-                        (long long)(atomicAdd((unsigned long long *)&A.w[s_hub[h]], (unsigned long long)0 - a) - a);
+                    long long *w = compact ? nwl : wl;  // only live heads were added up
+                    const long long nv = (long long)(atomicAdd((unsigned long long *)&w[rank_pos(rank_word(A.rank, s_hub[h]), s_hub[h])],
+                                                               (unsigned long long)0 - a) - a);
                     mindec = nv < mindec ? nv : mindec;
                     s_hlo[h] = 0;
                     s_hhi[h] = 0;
@@ -877,6 +1056,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
                 st.round = i;
                 st.n_min_rule += s_rd.minrule;
                 if (s_rd.compact) {
+                    s_moved = 1;
                     st.live_sel ^= 1;
                     st.live_len = s_rd.newSize;
                 }
@@ -894,6 +1074,19 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             }
             __syncthreads();
         }
+    }
+    // the survivors' weights by id again, for the tails (positions and ids share
+    // w after an even number of compactions, so those pass through w2)
+    if (s_st.size > 0 && s_moved) {
+        const long long L = s_st.live_len;
+        const long long j0 = split_at(L, b, G), j1 = split_at(L, b + 1, G);
+        const int *live = s_st.live_sel ? A.live1 : A.live0;
+        if (!s_st.live_sel) {
+            for (long long j = j0 + tid; j < j1; j += BULK_THREADS) A.w2[j] = A.w[j];
+            if (!grid_barrier(ctl, G, bar_target)) return;
+        }
+        for (long long j = j0 + tid; j < j1; j += BULK_THREADS)
+            if (live[j] >= 0) A.w[live[j]] = A.w2[j];
     }
     if (b == 0 && tid == 0) {
         const RoundState &st = s_st;
@@ -970,8 +1163,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tail_scan(PeelArgs A, long lon
 // pass 0: count live neighbours per live vertex; pass 1: fill local arcs
 template <int PASS>
 __global__ void __launch_bounds__(BULK_THREADS) k_tail_arcs(PeelArgs A) {
-    __shared__ long long s_base[WALK_WIN + 1];
-    __shared__ long long s_start[WALK_WIN + 1];
+    __shared__ WalkShared s_walk;
     __shared__ long long s_k0;
     const PeelCtl *c = A.ctl;
     if (!builds(c, 0)) return;
@@ -993,24 +1185,37 @@ __global__ void __launch_bounds__(BULK_THREADS) k_tail_arcs(PeelArgs A) {
     const int *col = A.g.col;
     const int *hubs = A.g.hubs;
     const long long *cw = A.g.cw;
-    const int *pr = A.pr;
+    const RankWord *rank = A.rank;
     const bool grp = c->status == ST_CLUSTER && A.tgrp != nullptr && A.cl_c > 0;
-    walk_arcs([=](long long k) { return tdeg[k]; },
-              [=](long long k) { return rp[live[k]]; }, L, e0, e1, k0, s_base, s_start,
-              [&](long long k, long long pos) {
-                  const int v = arc_head(col[pos], hubs);
-                  if (pr[v] != DUPIN_LIVE) return;
-                  if (PASS == 0) {  // per row (per row and owner for the cluster; k_tail_rowcnt adds them up)
-                      if (grp) atomicAdd(&A.tgrp[k * DUPIN_GRP_STRIDE + 1 + (A.loc[v] & (A.cl_c - 1))], 1u);
-                      else atomicAdd(&A.tcnt[k], 1);
-                  } else {
-                      const long long slot =
-                          grp ? (long long)atomicAdd(&A.tgrp[k * DUPIN_GRP_STRIDE + 1 + (A.loc[v] & (A.cl_c - 1))], 1u)
-                              : A.tlrp[k] + atomicAdd(&A.tfill[k], 1);
-                      A.tcol[slot] = A.loc[v];
-                      if (A.tcw) A.tcw[slot] = cw ? cw[pos] : DUPIN_Q_ONE;
-                  }
-              });
+    walk_arcs<BULK_THREADS, BUILD_ILP, true>(
+        [=](long long k) { return tdeg[k]; }, [=](long long k) { return rp[live[k]]; }, L, e0, e1, k0, s_walk,
+        [&](const long long (&k)[BUILD_ILP], const long long (&pos)[BUILD_ILP]) {
+            int v[BUILD_ILP], to[BUILD_ILP];
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) v[u] = pos[u] >= 0 ? col[pos[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) {
+                if (v[u] < 0) v[u] = hubs[-v[u] - 1];
+                if (pos[u] >= 0 && !((rank[v[u] >> 5].live >> (v[u] & 31)) & 1u)) v[u] = -1;
+                if (pos[u] < 0) v[u] = -1;
+            }
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) to[u] = v[u] >= 0 && (PASS || grp) ? A.loc[v[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < BUILD_ILP; u++) {
+                if (v[u] < 0) continue;
+                if (PASS == 0) {  // per row (per row and owner for the cluster; k_tail_rowcnt adds them up)
+                    if (grp) atomicAdd(&A.tgrp[k[u] * DUPIN_GRP_STRIDE + 1 + (to[u] & (A.cl_c - 1))], 1u);
+                    else atomicAdd(&A.tcnt[k[u]], 1);
+                } else {
+                    const long long slot =
+                        grp ? (long long)atomicAdd(&A.tgrp[k[u] * DUPIN_GRP_STRIDE + 1 + (to[u] & (A.cl_c - 1))], 1u)
+                            : A.tlrp[k[u]] + atomicAdd(&A.tfill[k[u]], 1);
+                    A.tcol[slot] = to[u];
+                    if (A.tcw) A.tcw[slot] = cw ? cw[pos[u]] : DUPIN_Q_ONE;
+                }
+            }
+        });
 }
 
 // For the cluster tail: each row's live-arc count, from its owner groups' counts
@@ -1174,7 +1379,7 @@ int peel_grid_size() {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_peel_bulk, BULK_THREADS, 0);
     if (occ < 1) occ = 1;
     if (occ > 2) occ = 2;
-    // the consumer starts of one round are staged in s_base (WALK_WIN + 1 entries)
+    // the consumer starts of one round are staged in the walk's window (WALK_WIN entries)
     return std::min(sms * occ, WALK_WIN);
 }
 
@@ -1246,8 +1451,8 @@ long long workspace_bytes(long long n, long long arcs, bool has_cw, const PeelPl
     const long long tail_cap = plan.hcap(), tr_cap = plan.tr_cap;
     const long long tarc = tail_arc_buffer(arcs, plan);
     long long b = 0;
-    // w, pr, live0, live1, stage_id, stage_start, stage_off, fstart, loc, mask; fbase
-    b += n * (8 + 4 + 4 + 4 + 4 + 8 + 8 + 8 + 4 + 1) + 8 * (n + 1);
+    // w, w2, pr, live0, live1, stage_start, stage_deg, fstart, loc, mask; fbase; rank
+    b += n * (8 + 8 + 4 + 4 + 4 + 8 + 4 + 8 + 4 + 1) + 8 * (n + 1) + (long long)sizeof(RankWord) * ((n + 31) / 32);
     b += 8 * (grid + 1) + (long long)sizeof(BlockPart) * grid + (long long)sizeof(PeelCtl);
     b += 32 * tr_cap;
     b += (tail_cap + 1) * (8 + 8 + 4 + 4 + 4 * DUPIN_GRP_STRIDE);
@@ -1257,10 +1462,10 @@ long long workspace_bytes(long long n, long long arcs, bool has_cw, const PeelPl
 
 void workspace_free(PeelWorkspace *ws, cudaStream_t s) {
     if (!ws) return;
-    void *ptrs[] = {ws->w, ws->pr, ws->live0, ws->live1, ws->stage_id, ws->stage_start, ws->stage_off,
+    void *ptrs[] = {ws->w, ws->pr, ws->w2, ws->live0, ws->live1, ws->stage_start, ws->stage_deg,
                     ws->fstart, ws->fbase, ws->cstart, ws->part, ws->ctl, ws->tr_f_hi, ws->tr_f_lo,
                     ws->tr_size, ws->tr_peeled, ws->loc, ws->tdeg, ws->tlrp, ws->tcnt, ws->tfill,
-                    ws->tgrp, ws->tbuf, ws->mask};
+                    ws->tgrp, ws->tbuf, ws->mask, ws->rank};
     for (void *q : ptrs) {
         if (!q) continue;
         if (ws->async) cudaFreeAsync(q, s);
@@ -1296,9 +1501,9 @@ PeelWorkspace *workspace_create(long long n, long long arcs, bool has_cw, const 
     A(&ws->pr, n);
     A(&ws->live0, n);
     A(&ws->live1, n);
-    A(&ws->stage_id, n);
+    A(&ws->w2, n);
     A(&ws->stage_start, n);
-    A(&ws->stage_off, n);
+    A(&ws->stage_deg, n);
     A(&ws->fstart, n);
     A(&ws->fbase, n + 1);
     A(&ws->cstart, ws->grid + 1);
@@ -1321,6 +1526,7 @@ PeelWorkspace *workspace_create(long long n, long long arcs, bool has_cw, const 
     if (has_cw) ws->tcw = (long long *)ws->tbuf;
     ws->tcol = (int *)(ws->tbuf + wbytes);
     A(&ws->mask, n);
+    A(&ws->rank, (n + 31) / 32);
     if (e != cudaSuccess) {
         workspace_free(ws, s);
         cudaGetLastError();
@@ -1427,9 +1633,11 @@ static PeelArgs make_args(const dupin_graph *g, const PeelWorkspace *ws, const d
     A.pr = ws->pr;
     A.live0 = ws->live0;
     A.live1 = ws->live1;
-    A.stage_id = ws->stage_id;
+    A.w2 = ws->w2;
+    A.rank = ws->rank;
+    A.stage_id = ws->loc;
     A.stage_start = ws->stage_start;
-    A.stage_off = ws->stage_off;
+    A.stage_deg = ws->stage_deg;
     A.fstart = ws->fstart;
     A.fbase = ws->fbase;
     A.cstart = ws->cstart;
@@ -1489,11 +1697,12 @@ __global__ void k_ctl_reset(PeelCtl *c) {
 // A follower of a batched call: the initial weights of the same graph and
 // metric copied from another workspace, the live state set up as the
 // initial-weight kernels would, and the sums f(V) and min w copied.
-__global__ void k_init_follow(long long n, const long long *src_w, long long *w, int *pr, int *live0) {
+__global__ void k_init_follow(long long n, const long long *src_w, long long *w, int *pr, int *live0, RankWord *rank) {
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
         w[u] = src_w[u];
         pr[u] = DUPIN_LIVE;
         live0[u] = (int)u;
+        if ((u & 31) == 0) rank[u >> 5] = RankWord{~0u, ~0u, (unsigned)u, 0};
     }
 }
 
@@ -1520,10 +1729,10 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
             int sms = 0, dev = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            k_init_follow<<<sms * 8, 256, 0, s>>>(g->n, init_from->w, ws->w, ws->pr, ws->live0);
+            k_init_follow<<<sms * 8, 256, 0, s>>>(g->n, init_from->w, ws->w, ws->pr, ws->live0, ws->rank);
             k_init_follow_ctl<<<1, 1, 0, s>>>(init_from->ctl, ws->ctl);
         } else {
-            rc = launch_init_weights(A.g, p->metric, ws->w, ws->pr, ws->live0, ws->ctl, false, s);
+            rc = launch_init_weights(A.g, p->metric, ws->w, ws->pr, ws->live0, ws->rank, ws->ctl, false, s);
             if (rc) return rc;
         }
         k_init_finish<<<1, 1, 0, s>>>(A, g->n);
@@ -1705,7 +1914,7 @@ int peel_finish(const dupin_graph *g, PeelWorkspace *ws, const dupin_params *p, 
 // initial weights (validated when 'check'), round 0, then all rounds in one CTA.
 int launch_small_graph_peel(const PeelArgs &A, int metric, bool check, cudaStream_t s) {
     k_ctl_reset<<<1, 1, 0, s>>>(A.ctl);
-    int rc = launch_init_weights(A.g, metric, A.w, A.pr, A.live0, A.ctl, check, s);
+    int rc = launch_init_weights(A.g, metric, A.w, A.pr, A.live0, nullptr, A.ctl, check, s);
     if (rc) return rc;
     k_init_finish<<<1, 1, 0, s>>>(A, A.g.n);
     PeelArgs B = A;

@@ -7,8 +7,9 @@
 #define BULK_WARPS (BULK_THREADS / 32)
 #define WALK_WIN 1024
 #ifndef BULK_ILP
-#define BULK_ILP 1  // arcs in flight per thread in the grid-wide expand (1 measured best)
+#define BULK_ILP 3  // arcs in flight per thread in the grid-wide expand
 #endif
+#define BUILD_ILP 4  // and in the tail builds
 #define INIT_THREADS 256
 #define INIT_WARPS (INIT_THREADS / 32)
 #ifndef INIT_UNROLL
@@ -97,19 +98,9 @@ __device__ __forceinline__ long long block_excl_scan(long long x, long long *s_w
     return before + incl - x;
 }
 
-// last t in [0, WALK_WIN] with s[t] <= x (s non-decreasing, s[0] <= x):
-// a fixed number of predicated steps, so that several searches interleave
-__device__ __forceinline__ int smem_last_le_fixed(const long long *s, long long x) {
-    static_assert((WALK_WIN & (WALK_WIN - 1)) == 0, "WALK_WIN: a power of two");
-    int t = 0;
-#pragma unroll
-    for (int step = WALK_WIN; step > 0; step >>= 1)
-        if (t + step <= WALK_WIN && s[t + step] <= x) t += step;
-    return t;
-}
-
 // last t in [0, n) with s[t] <= x (s non-decreasing, s[0] <= x)
-__device__ __forceinline__ int smem_last_le(const long long *s, int n, long long x) {
+template <class T>
+__device__ __forceinline__ int smem_last_le(const T *s, int n, T x) {
     int lo = 0, hi = n - 1;
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
@@ -121,30 +112,78 @@ __device__ __forceinline__ int smem_last_le(const long long *s, int n, long long
 
 // Walk the arcs [e0, e1) of a segmented arc space.  Entry k (0 <= k < U)
 // covers [base(k), base(k+1)) and its arcs sit at col positions start(k) + (x -
-// base(k)); base(U) is the total.  k0 must satisfy base(k0) <= e0.  The
-// block loads WALK_WIN entries at a time into shared memory and calls
-// fn(k, pos) once per arc, consecutive threads on consecutive arcs.
-template <class BaseF, class StartF, class ArcF>
-__device__ __forceinline__ void walk_arcs(BaseF base, StartF start, long long U, long long e0, long long e1,
-                                          long long k0, long long *s_base, long long *s_start, ArcF fn) {
+// base(k)); base(U) is the total.  k0 is the entry of arc e0.  EMPTY: entries may
+// be empty.  The block loads WALK_WIN entries at a time into shared memory; each
+// warp then takes 32 ILP consecutive arcs at a time and calls fn(k, pos) once
+// with the entries and positions of its lane's ILP arcs (pos < 0: none).  The
+// first arc's entry is found by two ballots; within 32 arcs, the entries that
+// start there set a bit each of one word, and a lane counts the bits up to its
+// own (a binary search per arc took ten dependent shared loads).
+struct WalkShared {
+    int base[WALK_WIN + 1];         // first arc of each entry, from the window's first arc on, cut off at WALK_FAR
+    long long off[WALK_WIN];        // position = off + arc (from the window's first arc on)
+    long long next;
+};
+#define WALK_FAR (1 << 30)
+
+template <int NT, int ILP, bool EMPTY, class BaseF, class StartF, class ArcF>
+__device__ __forceinline__ void walk_arcs(BaseF base, StartF start, long long U, long long e0, long long e1, long long k0,
+                                          WalkShared &S, ArcF fn) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned le = 0xffffffffu >> (31 - lane);
     long long e = e0, k = k0;
-    while (e < e1) {
+    while (e < e1) {  // block-uniform
         __syncthreads();
-        for (int t = threadIdx.x; t <= WALK_WIN; t += blockDim.x) {
-            long long idx = k + t;
-            s_base[t] = idx <= U ? base(idx) : kMaxLL;
-            s_start[t] = idx < U ? start(idx) : 0;
+        for (int t = threadIdx.x; t <= WALK_WIN; t += NT) {
+            const long long idx = k + t;
+            const long long b = idx <= U ? base(idx) : e + WALK_FAR;
+            S.base[t] = (int)(b < e ? 0 : (b - e < WALK_FAR ? b - e : WALK_FAR));
+            if (t < WALK_WIN) S.off[t] = idx < U ? start(idx) - (b - e) : 0;
         }
         __syncthreads();
-        long long wend = s_base[WALK_WIN];
-        long long hi = e1 < wend ? e1 : wend;
-        for (long long x = e + threadIdx.x; x < hi; x += blockDim.x) {
-            int t = smem_last_le(s_base, WALK_WIN, x);
-            fn(k + t, s_start[t] + (x - s_base[t]));
+        long long span = S.base[WALK_WIN];  // arcs the window covers, or WALK_FAR
+        if (span > e1 - e) span = e1 - e;
+        const int hi = (int)span;
+        for (int c = 32 * ILP * wid; c < hi; c += ILP * NT) {
+            const unsigned m1 = __ballot_sync(0xffffffffu, S.base[32 * lane] <= c);
+            const int g = 32 * (31 - __clz(m1));
+            const unsigned m2 = __ballot_sync(0xffffffffu, S.base[g + lane] <= c);
+            int t = g + 31 - __clz(m2);  // the entry of arc c
+            long long pos[ILP], ent[ILP];
+#pragma unroll
+            for (int u = 0; u < ILP; u++) {
+                const int x0 = c + 32 * u;
+                pos[u] = -1;
+                ent[u] = 0;
+                if (x0 < hi) {  // warp-uniform
+                    const int d = (t + 1 + lane <= WALK_WIN ? S.base[t + 1 + lane] : WALK_FAR) - x0;  // at least 1
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, d < 32 ? 1u << d : 0u);
+                    int mine = t + __popc(starts & le), next = t + __popc(__ballot_sync(0xffffffffu, d <= 32));
+                    if (EMPTY && __popc(starts) != __popc(__ballot_sync(0xffffffffu, d < 32))) {  // empty entries among them
+                        mine = smem_last_le(S.base, WALK_WIN, x0 + lane);
+                        next = smem_last_le(S.base, WALK_WIN, x0 + 32);
+                    }
+                    if (x0 + lane < hi) {
+                        pos[u] = S.off[mine] + (x0 + lane);
+                        ent[u] = k + mine;
+                    }
+                    t = next;
+                }
+            }
+            fn(ent, pos);
         }
-        int t2 = smem_last_le(s_base, WALK_WIN + 1, hi);
-        k += t2;
-        e = hi;
+        // the next window: the entry of arc e + hi
+        if (e + hi < e1) {
+            if (wid == 0) {
+                const unsigned m1 = __ballot_sync(0xffffffffu, S.base[32 * lane] <= hi);
+                const int g = 32 * (31 - __clz(m1));
+                const unsigned m2 = __ballot_sync(0xffffffffu, S.base[g + lane] <= hi);
+                if (lane == 0) S.next = k + g + 31 - __clz(m2) + (S.base[WALK_WIN] <= hi && g + 31 - __clz(m2) == WALK_WIN - 1 ? 1 : 0);
+            }
+            __syncthreads();
+            k = S.next;
+        }
+        e += hi;
     }
 }
 
