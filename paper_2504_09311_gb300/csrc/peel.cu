@@ -1,29 +1,31 @@
 // peel.cu -- Dupin's parallel batch peeling (Algorithm 2, Sec. 4.1) on sm_103a.
 //
 // One peel = four stages, all on the caller's stream:
-//  (a) initial peeling weights w_u(V) = a_u + sum_v c_uv: an arc-balanced
-//      segmented sum over the CSR (each warp streams a contiguous arc range,
-//      carries the open row across chunks, so a hub row costs one atomic per
-//      warp), then f(V) = sum_u (w_u + a_u) / 2 and min_u w_u;
-//  (b)-(c) the bulk rounds in one persistent cooperative kernel, three grid
-//      barriers per round:
-//        A  select: scan this block's slice of the live list, peel every u
-//           with w_u <= T_i (T_i = floor(k (D+N) f / (D |S|)), or the minimum
-//           live weight when T_i selects nobody); stage the frontier with one
-//           packed (count, arcs) shared atomic per warp;
+//  (a) initial peeling weights w_u(V) = a_u + sum_v c_uv from running sums
+//      over tiles of arc weights, then f(V) = sum_u (w_u + a_u) / 2 and
+//      min_u w_u;
+//  (b)-(c) the grid-wide rounds in one persistent cooperative kernel, three
+//      grid barriers per round (one more where a minimum-rule round compacts):
+//        A  select: scan this block's slice of the live list and its weights
+//           (kept by list position), peel every u with w_u <= T_i (T_i =
+//           floor(k (D+N) f / (D |S|)), or the minimum live weight when T_i
+//           selects nobody); stage the frontier with one packed (count, arcs)
+//           shared atomic per warp;
 //        B  place: prefix the per-block counts, write the frontier with its
 //           arc offsets, record where each consumer block's equal share of
-//           the round's arcs starts (merge path), compact the live list when
-//           it has halved;
-//        C  expand: walk this block's share of the frontier's arcs, subtract
-//           c_uv from every surviving neighbour with an int64 atomic, sum c
+//           the round's arcs starts (merge path), compact the live list, in
+//           id order, with its weights and rank words when it has halved;
+//        C  expand: walk this block's share of the frontier's arcs, read each
+//           neighbour's rank word (live? where in the list?), subtract c_uv
+//           from every surviving one's weight with an int64 atomic, sum c
 //           over arcs inside U_i, and take the minimum post-decrement weight
 //           (the next round's minimum-rule candidate);
 //        D  (every block, redundantly) f_i = f_{i-1} - (sum_{u in U} w_u -
 //           internal/2), |S_i|, the best prefix, the trace;
-//  (d) once |S| <= tail_cap: the live vertices' induced subgraph is built
-//      (local ids, live arcs only) and one CTA runs the remaining rounds with
-//      w and the vertex states in shared memory.
+//  (d) once |S| is small enough: the live vertices' induced subgraph is built
+//      (local ids, live arcs only) and one CTA, or one cluster of CTAs, runs
+//      the remaining rounds; where nearly every round left takes one vertex of
+//      a small dense core, the core goes into a matrix instead.
 // Every step is exact integer arithmetic, so the per-round sets, the trace
 // and the best set equal the single-threaded oracle's bit for bit.
 #include <cooperative_groups.h>
@@ -32,6 +34,7 @@
 #include <stdio.h>
 
 #include <algorithm>
+#include <atomic>
 #include <string>
 
 #include <chrono>
@@ -77,17 +80,15 @@ __global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *li
     }
 }
 
-// Arc-balanced segmented sum: w_u += sum of c over row u.  The arc range is
+// Loading a graph: w_u += sum of c over row u, with every arc checked (ids,
+// self-loops, weights, int64 overflow, rows strictly increasing, the symmetry
+// fingerprint, the or of all weights).  The arc range is
 // split evenly over all warps of the grid; each warp walks its range in
 // 32-arc chunks, finds each arc's row from 32 cached row ends (5 shuffle
 // steps), reduces rows within the chunk with a segmented scan and keeps the
 // open last row in registers, so a row spanning many chunks is flushed once
-// per warp.  The loads of INIT_UNROLL chunks are issued together; registers
-// are held to what 6 resident blocks per SM allow (measured 3% faster on
-// R-MAT-24 than the default budget).  CHECK also validates ids, self-loops
-// and int64 overflow.
-template <bool CHECK>
-__global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGraph g, long long *w, PeelCtl *ctl) {
+// per warp.  The loads of INIT_UNROLL chunks are issued together.
+__global__ void __launch_bounds__(INIT_THREADS) k_init_arcs(DevGraph g, long long *w, PeelCtl *ctl) {
     const int lane = threadIdx.x & 31;
     const long long NW = (long long)gridDim.x * INIT_WARPS;
     const long long W = blockIdx.x * (long long)INIT_WARPS + (threadIdx.x >> 5);
@@ -98,14 +99,14 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
     long long r = warp_search_last_le(g.rp, n, we0);  // row of the first arc
     long long carry_own = -1, carry_val = 0;
     bool bad = false;
-    // CHECK: rows strictly increasing (each arc against the next, across
+    // rows strictly increasing (each arc against the next, across
     // chunks through the last arc seen, across warps through the arc before
     // the range) and the symmetry fingerprint
     bool unsorted = false;
     unsigned long long fp = 0, wor = 0;
     long long prev_row = -1;
     int prev_col = 0;
-    if (CHECK && g.rp[r] < we0) {  // the range starts inside row r: compare with the arc before it
+    if (g.rp[r] < we0) {  // the range starts inside row r: compare with the arc before it
         prev_row = r;
         prev_col = g.col[we0 - 1];
     }
@@ -123,20 +124,20 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
     };
     long long r_end = g.rp[r + 1];  // end of row r
     long long lacc = 0;             // per-lane partial sum of row r over whole-row chunks
-    // one 32-arc chunk whose weights (and, with CHECK, heads) are already loaded
+    // one 32-arc chunk whose weights and heads are already loaded
     auto chunk = [&](const long long x0, const long long val, const int cvx) {
         const long long x = x0 + lane;
         const bool valid = x < we1;
-        if (CHECK && valid) {
+        if (valid) {
             if (cvx < 0 || cvx >= n || val < 0) bad = true;
             wor |= (unsigned long long)val;
         }
         // fast path: the whole chunk lies in row r (long rows, hubs)
         const long long cend = x0 + 32 < we1 ? x0 + 32 : we1;
         if (cend <= r_end) {
-            if (CHECK) check_chunk(r, cvx, val, x, valid);
-            if (CHECK && valid && cvx == r) bad = true;  // self-loop
-            if (CHECK && (unsigned long long)lacc + (unsigned long long)val < (unsigned long long)lacc) bad = true;
+            check_chunk(r, cvx, val, x, valid);
+            if (valid && cvx == r) bad = true;  // self-loop
+            if ((unsigned long long)lacc + (unsigned long long)val < (unsigned long long)lacc) bad = true;
             lacc += val;
             return;
         }
@@ -179,8 +180,8 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
             if (!__any_sync(0xffffffffu, owner < 0)) break;
             rr += 32;
         }
-        if (CHECK && valid && cvx == owner) bad = true;
-        if (CHECK) check_chunk(owner, cvx, val, x, valid);
+        if (valid && cvx == owner) bad = true;
+        check_chunk(owner, cvx, val, x, valid);
         // segmented inclusive scan by owner
         long long sv = val;
 #pragma unroll
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
             long long ov = __shfl_up_sync(0xffffffffu, sv, d);
             long long oo = __shfl_up_sync(0xffffffffu, owner, d);
             if (lane >= d && oo == owner) {
-                if (CHECK && (unsigned long long)sv + (unsigned long long)ov < (unsigned long long)sv) bad = true;
+                if ((unsigned long long)sv + (unsigned long long)ov < (unsigned long long)sv) bad = true;
                 sv += ov;
             }
         }
@@ -200,12 +201,8 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         const long long oL = __shfl_sync(0xffffffffu, owner, last);
         if (carry_own >= 0 && carry_own != o0) {
             if (lane == 0) {
-                if (CHECK) {
-                    unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-                    if (old + (unsigned long long)carry_val < old) bad = true;
-                } else {
-                    atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-                }
+                unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
+                if (old + (unsigned long long)carry_val < old) bad = true;
             }
             carry_own = -1;
             carry_val = 0;
@@ -213,12 +210,8 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         const long long add = (carry_own == o0) ? carry_val : 0;
         if (is_end && owner != oL) {
             long long tot = sv + (owner == o0 ? add : 0);
-            if (CHECK) {
-                unsigned long long old = atomicAdd((unsigned long long *)&w[owner], (unsigned long long)tot);
-                if (old + (unsigned long long)tot < old) bad = true;
-            } else {
-                atomicAdd((unsigned long long *)&w[owner], (unsigned long long)tot);
-            }
+            unsigned long long old = atomicAdd((unsigned long long *)&w[owner], (unsigned long long)tot);
+            if (old + (unsigned long long)tot < old) bad = true;
         }
         long long lastsum = __shfl_sync(0xffffffffu, sv, last);
         carry_val = lastsum + (oL == o0 ? add : 0);
@@ -234,7 +227,7 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         for (int u = 0; u < INIT_UNROLL; u++) {
             const long long x = xb + 32 * u + lane;
             vals[u] = x < we1 ? g.cw[x] : 0;
-            cvs[u] = (CHECK && x < we1) ? g.col[x] : 0;
+            cvs[u] = x < we1 ? g.col[x] : 0;
         }
 #pragma unroll
         for (int u = 0; u < INIT_UNROLL; u++)
@@ -254,22 +247,16 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
         }
     }
     if (carry_own >= 0 && lane == 0) {
-        if (CHECK) {
-            unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-            if (old + (unsigned long long)carry_val < old) bad = true;
-        } else {
-            atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-        }
+        unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
+        if (old + (unsigned long long)carry_val < old) bad = true;
     }
-    if (CHECK && __any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctl->init_overflow, 1);
-    if (CHECK) {
-        if (__any_sync(0xffffffffu, unsorted) && lane == 0) atomicExch(&ctl->check_unsorted, 1);
-        for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);  // wrapping sum
-        if (lane == 0 && fp) atomicAdd(&ctl->check_fp, fp);
-        const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)wor);
-        const unsigned oh = __reduce_or_sync(0xffffffffu, (unsigned)(wor >> 32));
-        if (lane == 0) atomicOr(&ctl->check_or, ((unsigned long long)oh << 32) | ol);
-    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctl->init_overflow, 1);
+    if (__any_sync(0xffffffffu, unsorted) && lane == 0) atomicExch(&ctl->check_unsorted, 1);
+    for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);  // wrapping sum
+    if (lane == 0 && fp) atomicAdd(&ctl->check_fp, fp);
+    const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)wor);
+    const unsigned oh = __reduce_or_sync(0xffffffffu, (unsigned)(wor >> 32));
+    if (lane == 0) atomicOr(&ctl->check_or, ((unsigned long long)oh << 32) | ol);
 }
 
 // The same sums without the checks, for peeling: tiles of IT_TILE arc weights
@@ -280,7 +267,8 @@ __global__ void __launch_bounds__(INIT_THREADS, CHECK ? 1 : 6) k_init_arcs(DevGr
 // store per row, in row order.  Rows that cross a tile's edge are added up with
 // atomics (w holds a_u from k_init_vertex).  Sums wrap like any 64-bit ones.
 // The arc-balanced form above finds each arc's row by shuffles and scans rows
-// in registers: issue-bound, 1.76 ms on R-MAT scale 24 (4.2 GB of weights).
+// in registers: issue-bound, 1.76 ms on R-MAT scale 24 (4.2 GB of weights); this
+// takes 1.22 ms (3.4 TB/s), held by the barriers between a tile's steps.
 #define IT_THREADS 256
 #define IT_ITEMS 8
 #define IT_TILE (IT_THREADS * IT_ITEMS)
@@ -436,13 +424,14 @@ int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, i
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int vgrid = sms * 8;
+    // as many blocks as there is work for (1,216 blocks over 150 vertices took 16 us)
+    const int vgrid = (int)std::max<long long>(1, std::min<long long>(sms * 8, (dg.n + 255) / 256));
     const bool isdg = metric == DUPIN_DG || dg.cw == nullptr;
     k_init_vertex<<<vgrid, 256, 0, s>>>(dg, isdg ? 1 : 0, w, pr, live0, rank, ctl);
     if (!isdg) {
         if (dg.arcs > 0) {
-            int agrid = sms * 8;
-            if (check) k_init_arcs<true><<<agrid, INIT_THREADS, 0, s>>>(dg, w, ctl);
+            const int agrid = (int)std::min<long long>(sms * 8, (dg.arcs + 255) / 256);
+            if (check) k_init_arcs<<<agrid, INIT_THREADS, 0, s>>>(dg, w, ctl);
             else k_init_tiles<<<(int)std::min<long long>(sms * 6, (dg.arcs + IT_TILE - 1) / IT_TILE), IT_THREADS, 0, s>>>(dg, w, ctl);
         }
         k_init_reduce<<<vgrid, 256, 0, s>>>(dg, w, ctl);
@@ -1346,25 +1335,38 @@ void launch_mask(const int *pr, long long n, long long best_round, uint8_t *mask
     k_mask_rounds<<<grid > 0 ? grid : 1, 256, 0, s>>>(pr, n, best_round, mask);
 }
 
-// best_mask[u] = (peel_round[u] > best_round)
+// best_mask[u] = (peel_round[u] > best_round) of a complete peel
 __global__ void k_finalize(const int *pr, long long n, const PeelCtl *ctl, uint8_t *mask) {
     const long long br = ctl->best_round;
+    if (ctl->error || ctl->status != ST_DONE) return;
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x)
         mask[u] = (long long)pr[u] > br ? 1 : 0;
+}
+
+void launch_finalize(const int *pr, long long n, const PeelCtl *ctl, uint8_t *mask, cudaStream_t s) {
+    k_finalize<<<(int)std::max<long long>(1, std::min<long long>(608, (n + 255) / 256)), 256, 0, s>>>(pr, n, ctl, mask);
 }
 
 // ------------------------------------------------------------------- host
 
 long long tail_cap_limit() {
+    // looked up once per device: a batch of thousands of graphs asks for every one
+    static std::atomic<long long> known[64];
     int dev = 0, smem = 0;
     cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64) {
+        const long long k = known[dev].load(std::memory_order_relaxed);
+        if (k) return k - 1;
+    }
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    // static shared memory of k_peel_tail is about 5 KB; 14 bytes per vertex
+    // static shared memory of k_peel_tail is about 3 KB; 14 bytes per vertex
     // plus padding to whole 64-vertex segments and 16 bytes per segment
     long long avail = (long long)smem - 8 * 1024 - 8 * TAIL_SEG - 32;
     long long cap = avail / (14 + 1);
     if (cap > 65535) cap = 65535;
-    return cap < 0 ? 0 : cap;
+    if (cap < 0) cap = 0;
+    if (smem > 0 && dev >= 0 && dev < 64) known[dev].store(cap + 1, std::memory_order_relaxed);
+    return cap;
 }
 
 long long tail_cap_default() {
@@ -1729,7 +1731,7 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
             int sms = 0, dev = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            k_init_follow<<<sms * 8, 256, 0, s>>>(g->n, init_from->w, ws->w, ws->pr, ws->live0, ws->rank);
+            k_init_follow<<<(int)std::max<long long>(1, std::min<long long>(sms * 8, (g->n + 255) / 256)), 256, 0, s>>>(g->n, init_from->w, ws->w, ws->pr, ws->live0, ws->rank);
             k_init_follow_ctl<<<1, 1, 0, s>>>(init_from->ctl, ws->ctl);
         } else {
             rc = launch_init_weights(A.g, p->metric, ws->w, ws->pr, ws->live0, ws->rank, ws->ctl, false, s);
@@ -1882,11 +1884,8 @@ int peel_finish(const dupin_graph *g, PeelWorkspace *ws, const dupin_params *p, 
     const cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     const long long n = g->n;
     if (r->best_mask && n > 0) {
-        int sms = 0, d = 0;
-        cudaGetDevice(&d);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, d);
         uint8_t *dst = dev ? r->best_mask : ws->mask;
-        k_finalize<<<sms * 4, 256, 0, s>>>(ws->pr, n, ws->ctl, dst);
+        launch_finalize(ws->pr, n, ws->ctl, dst, s);
         if (!dev) DUPIN_CUDA_TRY(cudaMemcpyAsync(r->best_mask, ws->mask, (size_t)n, cudaMemcpyDeviceToHost, s));
     }
     if (r->peel_round && n > 0)

@@ -436,7 +436,9 @@ def peel_batch(graphs: Sequence[Graph], params: Sequence[Params], want_rounds=Tr
     or a BatchBuffers (reusable: addresses computed once)."""
     k = len(graphs)
     G = np.fromiter((g.handle.value for g in graphs), dtype=np.uint64, count=k)
-    P = (Params * k)(*params)
+    raw = b"".join(map(bytes, params)) if all(type(p) is Params for p in params) else b""
+    # one copy for all of them (the array constructor takes 0.3 us each)
+    P = (Params * k).from_buffer_copy(raw) if k and len(raw) == k * ctypes.sizeof(Params) else (Params * k)(*params)
     if isinstance(buffers, BatchBuffers):
         keep, RA = buffers.keep, buffers.template.copy()
     else:
