@@ -181,19 +181,22 @@ typedef struct {
  * Scalars (always host): n_rounds R, best_round b (S_b = {u : peel_round[u]
  * > b}), |S_b|, f(S_b) as (hi, lo), g(S_b) as a double (value, not Q32.32),
  * how many rounds used the minimum-weight rule, how many rounds ran in the
- * grid-wide kernel (the rest ran in a tail), the tail's arc count (0 when
+ * grid-wide kernel before the first tail, the tail's arc count (0 when
  * the grid-wide rounds emptied S), with DUPIN_TIMING the device time of
  * each phase: [0] initial weights, [1] grid-wide rounds, [2] tail sub-graph
  * build, [3] tail rounds; and the CTAs of the tail that ran (1: the one-CTA
  * tail, 8 or 16: the cluster tail, 0: no tail).
  *
- * The tail: once the live set is small, one of two kernels finishes the
- * peel on the live sub-graph -- one CTA with the state in its shared memory
+ * The tail: once the live set is small, a kernel of one of two forms finishes
+ * the peel on the live sub-graph -- one CTA with the state in its shared memory
  * (live sets of at most about 14,900 vertices whose sub-graph has at most
  * 2^20 arcs), or a thread-block cluster of 8 or 16 CTAs with the state
  * spread over their shared memory (live sets of up to about 195,000
  * vertices).  Both give identical results; the flags DUPIN_TAIL_ONE_CTA and
- * DUPIN_TAIL_CLUSTER force one of them.
+ * DUPIN_TAIL_CLUSTER force one of them.  On graphs of more than 2^20 arcs with
+ * k(1+eps) < 2 a cluster continues on a matrix of the live vertices once that
+ * fits (also instead of one CTA, from 2^16 live arcs on), and on graphs of 2^27
+ * arcs and more it may give a peel back to the grid-wide kernel once.
  */
 typedef struct {
     uint8_t *best_mask;

@@ -320,7 +320,6 @@ extern "C" int dupin_graph_load(const dupin_graph_desc *d, void *stream, dupin_g
     }
     if (d->vertex_w) TRY(cudaMemcpyAsync(g->a, d->vertex_w, sizeof(long long) * (size_t)n, k, s));
     k_check_offsets<<<grid, 256, 0, s>>>(g->rp, n, arcs, bad);
-    if (has_w) k_check_nonneg<<<grid, 256, 0, s>>>(g->cw, arcs, bad);
     if (g->a) k_check_nonneg<<<grid, 256, 0, s>>>(g->a, n, bad);
     int hbad = 0;
     TRY(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -371,6 +370,11 @@ extern "C" int dupin_graph_load(const dupin_graph_desc *d, void *stream, dupin_g
             gfree(bad, s);
             return r2;
         }
+        if ((long long)hc.check_or < 0) {  // a weight with its sign bit set
+            graph_release(g);
+            gfree(bad, s);
+            return dupin_fail(DUPIN_ERR_INVALID_ARG, "invalid CSR: offsets, ids or weights out of range");
+        }
         if (hc.init_overflow) {
             graph_release(g);
             gfree(bad, s);
@@ -380,7 +384,7 @@ extern "C" int dupin_graph_load(const dupin_graph_desc *d, void *stream, dupin_g
                               "peeling weight >= 2^63");
         }
         // sorted rows without repeats, and symmetry: checked in the same pass
-        // (k_init_arcs with its checks on), read here once the ids are known valid
+        // (k_check_tiles), read here once the ids are known valid
         if (arcs > 0 && (hc.check_unsorted || hc.check_fp)) {
             graph_release(g);
             gfree(bad, s);

@@ -80,195 +80,17 @@ __global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *li
     }
 }
 
-// Loading a graph: w_u += sum of c over row u, with every arc checked (ids,
-// self-loops, weights, int64 overflow, rows strictly increasing, the symmetry
-// fingerprint, the or of all weights).  The arc range is
-// split evenly over all warps of the grid; each warp walks its range in
-// 32-arc chunks, finds each arc's row from 32 cached row ends (5 shuffle
-// steps), reduces rows within the chunk with a segmented scan and keeps the
-// open last row in registers, so a row spanning many chunks is flushed once
-// per warp.  The loads of INIT_UNROLL chunks are issued together.
-__global__ void __launch_bounds__(INIT_THREADS) k_init_arcs(DevGraph g, long long *w, PeelCtl *ctl) {
-    const int lane = threadIdx.x & 31;
-    const long long NW = (long long)gridDim.x * INIT_WARPS;
-    const long long W = blockIdx.x * (long long)INIT_WARPS + (threadIdx.x >> 5);
-    const long long A = g.arcs, n = g.n;
-    const long long we0 = split_at(A, W, NW);
-    const long long we1 = split_at(A, W + 1, NW);
-    if (we0 >= we1) return;
-    long long r = warp_search_last_le(g.rp, n, we0);  // row of the first arc
-    long long carry_own = -1, carry_val = 0;
-    bool bad = false;
-    // rows strictly increasing (each arc against the next, across
-    // chunks through the last arc seen, across warps through the arc before
-    // the range) and the symmetry fingerprint
-    bool unsorted = false;
-    unsigned long long fp = 0, wor = 0;
-    long long prev_row = -1;
-    int prev_col = 0;
-    if (g.rp[r] < we0) {  // the range starts inside row r: compare with the arc before it
-        prev_row = r;
-        prev_col = g.col[we0 - 1];
-    }
-    auto check_chunk = [&](const long long own, const int cvx, const long long val, const long long x,
-                           const bool valid) {
-        const int ncol = __shfl_down_sync(0xffffffffu, cvx, 1);
-        const long long nown = __shfl_down_sync(0xffffffffu, own, 1);
-        if (valid && lane < 31 && x + 1 < we1 && nown == own && ncol <= cvx) unsorted = true;
-        if (lane == 0 && valid && own == prev_row && cvx <= prev_col) unsorted = true;
-        if (valid) fp += sym_mix(g.key, own, cvx, val) - sym_mix(g.key, cvx, own, val);
-        const unsigned vm = __ballot_sync(0xffffffffu, valid);
-        const int lst = 31 - __clz(vm);
-        prev_row = __shfl_sync(0xffffffffu, own, lst);
-        prev_col = __shfl_sync(0xffffffffu, cvx, lst);
-    };
-    long long r_end = g.rp[r + 1];  // end of row r
-    long long lacc = 0;             // per-lane partial sum of row r over whole-row chunks
-    // one 32-arc chunk whose weights and heads are already loaded
-    auto chunk = [&](const long long x0, const long long val, const int cvx) {
-        const long long x = x0 + lane;
-        const bool valid = x < we1;
-        if (valid) {
-            if (cvx < 0 || cvx >= n || val < 0) bad = true;
-            wor |= (unsigned long long)val;
-        }
-        // fast path: the whole chunk lies in row r (long rows, hubs)
-        const long long cend = x0 + 32 < we1 ? x0 + 32 : we1;
-        if (cend <= r_end) {
-            check_chunk(r, cvx, val, x, valid);
-            if (valid && cvx == r) bad = true;  // self-loop
-            if ((unsigned long long)lacc + (unsigned long long)val < (unsigned long long)lacc) bad = true;
-            lacc += val;
-            return;
-        }
-        // leaving row r inside this chunk: fold the lanes' partials into the carry
-        {
-            long long sum = warp_sum64(lacc);
-            sum = __shfl_sync(0xffffffffu, sum, 0);
-            lacc = 0;
-            if (sum != 0) {
-                if (carry_own == r) carry_val += sum;
-                else {
-                    if (carry_own >= 0 && lane == 0)
-                        atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-                    carry_own = r;
-                    carry_val = sum;
-                }
-            }
-        }
-        // Row of each lane's arc: with the 32 row ends rp[rr+1 .. rr+32] held
-        // one per lane, a lane whose arc x has rp[rr] <= x < rp[rr+32] lies in
-        // row rr + #{j : rp[rr+1+j] <= x} (5 shuffle steps).  Lanes further
-        // out wait while the window moves on by 32 rows.
-        long long owner = valid ? -1 : kMaxLL;
-        long long rr = r;
-        for (;;) {
-            const long long idx = rr + 1 + lane;
-            const long long bj = idx <= n ? g.rp[idx] : kMaxLL;
-            // count in [0, 32]: 33 outcomes, so six halving steps
-            int lo = 0, hi = 32;
-#pragma unroll
-            for (int s = 0; s < 6; s++) {
-                const int mid = (lo + hi) >> 1;
-                const long long bm = __shfl_sync(0xffffffffu, bj, mid & 31);
-                if (lo < hi) {
-                    if (bm <= x) lo = mid + 1;
-                    else hi = mid;
-                }
-            }
-            if (owner < 0 && lo < 32) owner = rr + lo;
-            if (!__any_sync(0xffffffffu, owner < 0)) break;
-            rr += 32;
-        }
-        if (valid && cvx == owner) bad = true;
-        check_chunk(owner, cvx, val, x, valid);
-        // segmented inclusive scan by owner
-        long long sv = val;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            long long ov = __shfl_up_sync(0xffffffffu, sv, d);
-            long long oo = __shfl_up_sync(0xffffffffu, owner, d);
-            if (lane >= d && oo == owner) {
-                if ((unsigned long long)sv + (unsigned long long)ov < (unsigned long long)sv) bad = true;
-                sv += ov;
-            }
-        }
-        long long on = __shfl_down_sync(0xffffffffu, owner, 1);
-        const unsigned vmask = __ballot_sync(0xffffffffu, valid);
-        const int last = 31 - __clz(vmask);
-        const bool is_end = valid && (lane == last || on != owner);
-        const long long o0 = __shfl_sync(0xffffffffu, owner, 0);
-        const long long oL = __shfl_sync(0xffffffffu, owner, last);
-        if (carry_own >= 0 && carry_own != o0) {
-            if (lane == 0) {
-                unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-                if (old + (unsigned long long)carry_val < old) bad = true;
-            }
-            carry_own = -1;
-            carry_val = 0;
-        }
-        const long long add = (carry_own == o0) ? carry_val : 0;
-        if (is_end && owner != oL) {
-            long long tot = sv + (owner == o0 ? add : 0);
-            unsigned long long old = atomicAdd((unsigned long long *)&w[owner], (unsigned long long)tot);
-            if (old + (unsigned long long)tot < old) bad = true;
-        }
-        long long lastsum = __shfl_sync(0xffffffffu, sv, last);
-        carry_val = lastsum + (oL == o0 ? add : 0);
-        carry_own = oL;
-        r = oL;  // the next chunk starts in this row or later
-        r_end = g.rp[r + 1];
-    };
-    // INIT_UNROLL chunks per step: their loads are issued before any is processed
-    for (long long xb = we0; xb < we1; xb += 32 * INIT_UNROLL) {
-        long long vals[INIT_UNROLL];
-        int cvs[INIT_UNROLL];
-#pragma unroll
-        for (int u = 0; u < INIT_UNROLL; u++) {
-            const long long x = xb + 32 * u + lane;
-            vals[u] = x < we1 ? g.cw[x] : 0;
-            cvs[u] = x < we1 ? g.col[x] : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < INIT_UNROLL; u++)
-            if (xb + 32 * u < we1) chunk(xb + 32 * u, vals[u], cvs[u]);
-    }
-    {
-        long long sum = warp_sum64(lacc);
-        sum = __shfl_sync(0xffffffffu, sum, 0);
-        if (sum != 0) {
-            if (carry_own == r) carry_val += sum;
-            else {
-                if (carry_own >= 0 && lane == 0)
-                    atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-                carry_own = r;
-                carry_val = sum;
-            }
-        }
-    }
-    if (carry_own >= 0 && lane == 0) {
-        unsigned long long old = atomicAdd((unsigned long long *)&w[carry_own], (unsigned long long)carry_val);
-        if (old + (unsigned long long)carry_val < old) bad = true;
-    }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctl->init_overflow, 1);
-    if (__any_sync(0xffffffffu, unsorted) && lane == 0) atomicExch(&ctl->check_unsorted, 1);
-    for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);  // wrapping sum
-    if (lane == 0 && fp) atomicAdd(&ctl->check_fp, fp);
-    const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)wor);
-    const unsigned oh = __reduce_or_sync(0xffffffffu, (unsigned)(wor >> 32));
-    if (lane == 0) atomicOr(&ctl->check_or, ((unsigned long long)oh << 32) | ol);
-}
-
-// The same sums without the checks, for peeling: tiles of IT_TILE arc weights
+// w_u += sum of c over row u, for peeling: tiles of IT_TILE arc weights
 // arrive in shared memory by bulk copies, two buffers per block; a block scan
 // turns a tile into its running sums (a thread takes eight neighbours, reading
 // its four 16-byte pieces in an order that spreads a quarter-warp over the
 // banks), and each row inside the tile is the difference of two of them: a
 // store per row, in row order.  Rows that cross a tile's edge are added up with
 // atomics (w holds a_u from k_init_vertex).  Sums wrap like any 64-bit ones.
-// The arc-balanced form above finds each arc's row by shuffles and scans rows
-// in registers: issue-bound, 1.76 ms on R-MAT scale 24 (4.2 GB of weights); this
-// takes 1.22 ms (3.4 TB/s), held by the barriers between a tile's steps.
+// A form with the arcs split evenly over warps, each arc's row found by
+// shuffles and rows scanned in registers, was issue-bound: 1.76 ms on R-MAT
+// scale 24 (4.2 GB of weights); this takes 1.22 ms (3.4 TB/s), held by the
+// barriers between a tile's steps.
 #define IT_THREADS 256
 #define IT_ITEMS 8
 #define IT_TILE (IT_THREADS * IT_ITEMS)
@@ -280,6 +102,19 @@ __device__ __forceinline__ void it_load(long long *buf, const long long *src, un
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d), "l"(src),
                  "r"(bytes), "r"(m)
                  : "memory");
+}
+
+// false if the copy has not arrived within the limit
+static __device__ __forceinline__ bool it_wait(unsigned long long *mb, unsigned parity) {
+    const unsigned m = (unsigned)__cvta_generic_to_shared(mb);
+    unsigned done = 0;
+    for (long long it = 0; !done && it <= DUPIN_SPIN_LIMIT; it++)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(m), "r"(parity)
+            : "memory");
+    return done != 0;
 }
 
 __global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long *w, PeelCtl *ctl) {
@@ -313,24 +148,8 @@ __global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long
         long long *P = s_buf[k];
         const long long t0 = t * IT_TILE;
         const int len = (int)(A - t0 < IT_TILE ? A - t0 : IT_TILE);
-        bool bad = false;
-        {
-            const unsigned m = (unsigned)__cvta_generic_to_shared(&s_mb[k]);
-            unsigned done = 0;
-            for (long long it = 0; !done; it++) {
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, "
-                    "p;\n\t}"
-                    : "=r"(done)
-                    : "r"(m), "r"(parity)
-                    : "memory");
-                if (!done && it > DUPIN_SPIN_LIMIT) {  // a lost copy: cannot happen; give up rather than hang
-                    bad = true;
-                    break;
-                }
-            }
-        }
-        if (__syncthreads_or(bad)) {
+        if (__syncthreads_or(!it_wait(&s_mb[k], parity))) {  // a lost copy: cannot happen; give up rather than hang
+            if (t + 1 < T1) it_wait(&s_mb[k ^ 1], (unsigned)(((t + 1 - T0) >> 1) & 1));  // the copy still in flight
             if (tid == 0) set_error(ctl, DUPIN_ERR_TIMEOUT);
             return;
         }
@@ -396,6 +215,171 @@ __global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long
     }
 }
 
+// Loading a graph: the same sums by the same tiles, with every arc checked (ids,
+// self-loops, weights, w_u < 2^63, rows strictly increasing, the symmetry
+// fingerprint, the or of all weights).  The caller's arrays may be aligned to
+// their elements only, so plain coalesced loads fill the tile.  Each row that
+// starts in the tile marks its first arc; a running maximum over the marks gives
+// every arc its row.  Sums are 64-bit differences; a tile with a weight of 2^52
+// or more, whose sums could wrap, first forms the sums of the weights' upper 32
+// bits the same way: a row whose upper sum reaches 2^31 is too heavy, any other
+// cannot wrap.  Bound by issue: four 64-bit finalisers per arc for the
+// fingerprint.  16.7 million arcs in short rows take 167 us; arcs split evenly
+// over warps with rows found by shuffles took 304 us, and 54 us more for a pass
+// of its own over the weights' signs.
+__global__ void __launch_bounds__(IT_THREADS, 4) k_check_tiles(DevGraph g, long long *w, PeelCtl *ctl) {
+    __shared__ __align__(16) long long P[IT_TILE];
+    __shared__ __align__(16) int s_col[IT_TILE], s_own[IT_TILE];
+    __shared__ long long s_w[IT_THREADS / 32], s_row;
+    __shared__ int s_top[IT_THREADS / 32], s_prev;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const long long A = g.arcs, n = g.n;
+    const long long tiles = (A + IT_TILE - 1) / IT_TILE;
+    const long long T0 = split_at(tiles, blockIdx.x, gridDim.x), T1 = split_at(tiles, blockIdx.x + 1, gridDim.x);
+    if (T0 >= T1) return;
+    if (tid < 32) {
+        const long long r = warp_search_last_le(g.rp, n, T0 * IT_TILE);  // the row of the first arc (the last of equal starts)
+        if (lane == 0) s_row = r;
+    }
+    __syncthreads();
+    long long r0 = s_row;
+    bool bad = false, unsorted = false;
+    unsigned long long fp = 0, wor = 0;
+    for (long long t = T0; t < T1; t++) {
+        const long long t0 = t * IT_TILE;
+        const int len = (int)(A - t0 < IT_TILE ? A - t0 : IT_TILE);
+        const long long t1 = t0 + len;
+        long long x[IT_ITEMS];
+        int cv[IT_ITEMS];
+#pragma unroll
+        for (int i = 0; i < IT_ITEMS; i++) {
+            const int at = i * IT_THREADS + tid;
+            x[i] = at < len ? g.cw[t0 + at] : 0;
+            cv[i] = at < len ? g.col[t0 + at] : 0;
+        }
+        unsigned long long o = 0;
+#pragma unroll
+        for (int i = 0; i < IT_ITEMS; i++) {
+            const int at = i * IT_THREADS + tid;
+            o |= (unsigned long long)x[i];
+            if (cv[i] < 0 || cv[i] >= n || x[i] < 0) bad = true;
+            P[at] = x[i];
+            s_col[at] = cv[i];
+            s_own[at] = 0;
+        }
+        if (tid == 0) s_prev = t0 > 0 ? g.col[t0 - 1] : -1;
+        wor |= o;
+        const int wide = __syncthreads_or((o >> 52) != 0);
+        // this thread's eight arcs: piece c at arcs 8 tid + 2 c
+        longlong2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int c = (q + (tid >> 1)) & 3;
+            const longlong2 y = *(const longlong2 *)&P[IT_ITEMS * tid + 2 * c];
+#pragma unroll
+            for (int z = 0; z < 4; z++)
+                if (c == z) v[z] = y;
+        }
+        for (int upper = wide ? 1 : 0; upper >= 0; upper--) {
+            const int shift = upper ? 32 : 0;
+            longlong2 u[4];
+            long long sum = 0;
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                u[c].x = sum;
+                u[c].y = sum + (long long)((unsigned long long)v[c].x >> shift);
+                sum = u[c].y + (long long)((unsigned long long)v[c].y >> shift);
+            }
+            long long total;
+            const long long before = block_excl_scan<IT_THREADS / 32>(sum, s_w, total);  // P is read by now
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int c = (q + (tid >> 1)) & 3;
+                longlong2 y;
+#pragma unroll
+                for (int z = 0; z < 4; z++)
+                    if (c == z) y = u[z];
+                y.x += before;
+                y.y += before;
+                *(longlong2 *)&P[IT_ITEMS * tid + 2 * c] = y;
+            }
+            __syncthreads();
+            // rows that start before the tile's end, from the one holding its first arc on
+            for (long long rb = r0;; rb += IT_THREADS) {
+                const long long r = rb + tid;
+                long long b = t1, e = t1;
+                if (r < n) {
+                    b = g.rp[r];
+                    e = g.rp[r + 1];
+                }
+                if (b < t1) {
+                    const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
+                    if (hi > lo) {
+                        const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
+                        if (upper) {
+                            if (s >= 1LL << 31) bad = true;
+                        } else {
+                            s_own[lo - t0] = (int)(r - r0);
+                            if (b >= t0 && e <= t1) {
+                                w[r] = s + (g.a ? g.a[r] : 0);  // below 2^64: k_init_reduce sees the sign
+                            } else {
+                                const unsigned long long old = atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
+                                if (old + (unsigned long long)s < old) bad = true;
+                            }
+                        }
+                    }
+                    if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
+                }
+                if (__syncthreads_or(r >= n || b >= t1)) break;
+            }
+        }
+        // the row of every arc, and its checks
+        int own[IT_ITEMS], col[IT_ITEMS];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            *(int4 *)&own[4 * h] = *(const int4 *)&s_own[IT_ITEMS * tid + 4 * h];
+            *(int4 *)&col[4 * h] = *(const int4 *)&s_col[IT_ITEMS * tid + 4 * h];
+        }
+        int top = 0;
+#pragma unroll
+        for (int i = 0; i < IT_ITEMS; i++) top = own[i] > top ? own[i] : top;
+        int incl = top;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d && y > incl) incl = y;
+        }
+        if (lane == 31) s_top[wid] = incl;
+        int cur = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) cur = 0;
+        __syncthreads();
+        for (int i = 0; i < wid; i++) cur = s_top[i] > cur ? s_top[i] : cur;
+        int prev = tid ? s_col[IT_ITEMS * tid - 1] : s_prev;
+#pragma unroll
+        for (int i = 0; i < IT_ITEMS; i++) {
+            if (IT_ITEMS * tid + i >= len) break;
+            // a row's first arc: marked, or the tile's first where the row of r0 starts there
+            const bool first = own[i] > 0 || (tid == 0 && i == 0 && g.rp[r0] >= t0);
+            if (own[i] > 0) cur = own[i];
+            const long long r = r0 + cur;
+            const long long c = (i & 1) ? v[i >> 1].y : v[i >> 1].x;
+            if (col[i] == r) bad = true;
+            if (!first && prev >= col[i]) unsorted = true;
+            fp += sym_mix(g.key, r, col[i], c) - sym_mix(g.key, col[i], r, c);
+            prev = col[i];
+        }
+        r0 = s_row;
+        __syncthreads();  // the tile is read; s_row too
+    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicExch(&ctl->init_overflow, 1);
+    if (__any_sync(0xffffffffu, unsorted) && lane == 0) atomicExch(&ctl->check_unsorted, 1);
+    for (int d = 16; d > 0; d >>= 1) fp += __shfl_down_sync(0xffffffffu, fp, d);  // wrapping sum
+    if (lane == 0 && fp) atomicAdd(&ctl->check_fp, fp);
+    const unsigned ol = __reduce_or_sync(0xffffffffu, (unsigned)wor);
+    const unsigned oh = __reduce_or_sync(0xffffffffu, (unsigned)(wor >> 32));
+    if (lane == 0) atomicOr(&ctl->check_or, ((unsigned long long)oh << 32) | ol);
+}
+
 // sum over u of (w_u + a_u) and min w (DW/FD)
 __global__ void k_init_reduce(DevGraph g, const long long *w, PeelCtl *ctl) {
     unsigned long long lo = 0, hi = 0;
@@ -430,9 +414,9 @@ int launch_init_weights(const DevGraph &dg, int metric, long long *w, int *pr, i
     k_init_vertex<<<vgrid, 256, 0, s>>>(dg, isdg ? 1 : 0, w, pr, live0, rank, ctl);
     if (!isdg) {
         if (dg.arcs > 0) {
-            const int agrid = (int)std::min<long long>(sms * 8, (dg.arcs + 255) / 256);
-            if (check) k_init_arcs<<<agrid, INIT_THREADS, 0, s>>>(dg, w, ctl);
-            else k_init_tiles<<<(int)std::min<long long>(sms * 6, (dg.arcs + IT_TILE - 1) / IT_TILE), IT_THREADS, 0, s>>>(dg, w, ctl);
+            const int agrid = (int)std::min<long long>(sms * 6, (dg.arcs + IT_TILE - 1) / IT_TILE);
+            if (check) k_check_tiles<<<agrid, IT_THREADS, 0, s>>>(dg, w, ctl);
+            else k_init_tiles<<<agrid, IT_THREADS, 0, s>>>(dg, w, ctl);
         }
         k_init_reduce<<<vgrid, 256, 0, s>>>(dg, w, ctl);
     }

@@ -10,11 +10,6 @@
 #define BULK_ILP 3  // arcs in flight per thread in the grid-wide expand
 #endif
 #define BUILD_ILP 4  // and in the tail builds
-#define INIT_THREADS 256
-#define INIT_WARPS (INIT_THREADS / 32)
-#ifndef INIT_UNROLL
-#define INIT_UNROLL 4  // 32-arc chunks whose loads a warp issues together in the initial weights
-#endif
 #ifndef TAIL_THREADS
 #define TAIL_THREADS 256
 #endif
