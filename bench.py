@@ -7,7 +7,7 @@ b = c = 0.19, self-loops dropped and pairs merged: 260,377,346 edges) with
 Fraudar weights c = 1/ln(d_obj + 5) in Q32.32, peeled with the FD and the DG
 metric at the threshold (1 + eps) g(S) (k_mult = 1, eps = 1/10).  One step =
 the two peels of the whole hot path (initial weights, grid-wide rounds, tail
-sub-graph, tail rounds on one CTA or a thread-block cluster) in one batched
+sub-graph or matrix, tail rounds on one CTA or a thread-block cluster) in one batched
 call.  Beside it (not the headline): the same graph at k_mult = 2 and the DW
 metric (c uniform in 1..100, a uniform in 0..10) at k_mult = 1.
 
@@ -482,9 +482,25 @@ def run_reference(args, wl, rank, world):
 
 
 def kernel_of(phase: str, tail_ctas: int) -> str:
-    return {"init": "k_init_vertex+k_init_arcs+k_init_reduce", "bulk": "k_peel_bulk",
+    # the clusters' tail phase also holds the dense tail's build and, on graphs of
+    # 2^27 arcs and more, grid-wide rounds that a cluster tail gave back
+    return {"init": "k_init_vertex+k_init_tiles+k_init_reduce", "bulk": "k_peel_bulk",
             "build": "k_tail_prep+k_tail_scan+k_tail_arcs+k_tail_rowcnt+k_tail_grp",
-            "tail": "k_peel_cluster" if tail_ctas > 1 else "k_peel_tail"}[phase]
+            "tail": "k_peel_cluster+k_peel_dense" if tail_ctas > 1 else "k_peel_tail"}[phase]
+
+
+def launches_of(metric: str, eps, k: int, arcs: int) -> int:
+    """Kernels of one peel: control reset, initial weights (DG: one kernel; FD/DW: three), the set-up's
+    finish, the grid-wide rounds, the tail build (prep, two scans, two arc passes, row counts and owner
+    groups), the one-CTA and the cluster tail and the final mask; where the minimum rule can fire, the
+    dense tail (prep, scan, clear, fill, rounds) and on large graphs all of that again for a peel that
+    the cluster tail gives back.  Stages whose turn it is not return at once."""
+    n = 14 if metric == "dg" else 16
+    if k * (eps[1] + eps[0]) < 2 * eps[1] and arcs > 1 << 20:
+        n += 5
+        if arcs >= 1 << 27:
+            n += 1 + 7 + 2 + 5
+    return n
 
 
 def side_runs(dupin, g, dg, stream, wl, reps=3):
@@ -717,11 +733,6 @@ def main():
         cpu = cpu_baseline(g, metric_b, eps_b, k)
         cpu_par = cpu_parallel_baseline(g, metric_b, eps_b, k)
 
-    # kernels per peel: control reset, initial weights (DG: one kernel; FD/DW: three), the
-    # set-up's finish, the grid-wide rounds, the tail build (prep, two scans, two arc passes,
-    # row counts and owner groups), the one-CTA tail and the cluster tail (one of the two
-    # returns at once), and the final mask
-    launches_per_peel = {"dg": 14, "fd": 16, "dw": 16}
     line = {
         "metric": "edges peeled/s", "value": value, "unit": "edges/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -736,8 +747,7 @@ def main():
         "cpu_baseline": cpu,
         "cpu_parallel_baseline": cpu_par,
         "e2e": e2e,
-        # (+ one note per pair of the call's large peels: an earlier peel's tail kind for a later one)
-        "gpu_launches": (sum(launches_per_peel[m] for m, _ in peels) + len(peels) * (len(peels) - 1) // 2) * args.steps,
+        "gpu_launches": sum(launches_of(m, e, k, 2 * g.m) for m, e in peels) * args.steps,
         "clocks": clocks.summary(),
         "side": side,
         "batched": batched,
