@@ -922,8 +922,8 @@ static cudaStream_t tail_stream(int dev, size_t q) {
 // sets).  The initial weights are computed once per graph and metric; the
 // grid-wide stages run one after another on 'stream' (each is a
 // cooperative launch); each peel's tail sub-graph is built on 'stream' and
-// its one-CTA tail runs on a stream of its own, so the latency-bound tails,
-// one SM each, run side by side.  A graph that appears several times gets
+// its tail runs on a stream of its own, so the latency-bound tails, one SM or
+// one cluster each, run side by side.  A graph that appears several times gets
 // one cached workspace per appearance.
 static int peel_large_concurrent(dupin_graph *const *graphs, const dupin_params *params, dupin_result *results,
                                  const std::vector<int64_t> &idx, cudaStream_t s) {
@@ -1007,7 +1007,13 @@ static int peel_large_concurrent(dupin_graph *const *graphs, const dupin_params 
     // A peel that its cluster tail gave back runs its grid-wide rounds again on
     // 's' (one cooperative launch at a time), on the SMs that no other peel's
     // tail may hold, and its tails again on its own stream; with many peels,
-    // one after another once every tail is done.
+    // one after another once every tail is done.  They wait for the whole first
+    // tail stage, the dense tail's launches among them: those read the status
+    // that the second grid-wide rounds write, and a cluster launch can sit in
+    // its queue for as long as a cooperative grid holds the SMs.  (Queued before
+    // the next peel's grid-wide rounds, which slow the cluster tail beside them,
+    // the second stage won what that peel lost: 42.9 against 43.2 ms for FD and
+    // DG on R-MAT scale 24, 44.2 against 43.9 for DG and FD.)
     for (size_t q = 0; q < k && rc == DUPIN_OK && !overlap; q++) {
         cudaError_t e = cudaStreamWaitEvent(s, ev[2 * q + 1], 0);
         if (e != cudaSuccess) rc = dupin_cuda_fail(e, "tail stream join");
