@@ -49,6 +49,12 @@
 // values, so all CTAs leave together; a last barrier keeps every CTA's
 // shared memory alive until no other CTA can read it.  All arithmetic is
 // exact integer arithmetic, identical to the one-CTA tail's.
+//
+// The loop may end before the live set is empty: after a minimum-rule round
+// that leaves few enough vertices for the dense tail's matrix, and, on the
+// largest graphs, after a round by threshold of many vertices, whose expand
+// runs faster on the whole GPU.  The survivors' weights and live bits then go
+// back to memory, by id, for the next stage.
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
