@@ -306,7 +306,9 @@ int dupin_batch_tune(dupin_graph *const *graphs, const dupin_params *params, int
  * process whose allocator owns the device).  It runs the same peel as
  * dupin_peel on a graph of at most DUPIN_NOALLOC_MAX_N vertices given as a
  * symmetric CSR in DEVICE memory (row_ptr[n+1] int64, col_idx[row_ptr[n]]
- * int32, arc_w Q32.32 or NULL for DG, vertex_w or NULL), writes peel_round[n]
+ * int32, arc_w Q32.32 or NULL for DG, vertex_w or NULL; a row may be in any
+ * order and may hold a neighbour more than once, each arc then counting by
+ * itself), writes peel_round[n]
  * (device), the scalars of *result, and -- when non-NULL -- result->best_mask
  * and result->trace_* (device pointers, trace_cap entries).  It calls no
  * cudaMalloc, cudaFree or allocating library routine: its working state is

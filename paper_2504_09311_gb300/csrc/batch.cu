@@ -273,6 +273,7 @@ __device__ __forceinline__ void cta_peel_one(const CtaJob &J, unsigned char *sme
         S.use_min = J.use_min;
         S.gpo = J.gpo;
         S.lpo = J.lpo;
+        S.repeats = 0;  // the loader refuses them
         S.tr_f_hi = J.tr_f_hi;
         S.tr_f_lo = J.tr_f_lo;
         S.tr_size = J.tr_size;

@@ -208,6 +208,7 @@ struct PeelArgs {
     int desz, dshift;
     long long tail_smem;  // dynamic shared memory of the one-CTA tail
     int again;          // the cluster tail may give a collapsing graph back to the grid-wide rounds
+    int repeats;        // rows not checked to be strictly increasing: one may hold a head more than once
     long long dcap;
 };
 

@@ -17,9 +17,10 @@
 //
 //  - Warp form, for the minimum-rule rounds of one vertex that make up most of
 //    a weighted peel with k(1+eps) < 2: warp 0 runs round after round alone,
-//    without barriers, while the others wait.  The removed vertex's heads are
-//    distinct, so its decrements are plain loads and stores, SOLO_ILP chunks of
-//    32 arcs in flight.  It hands back to the block at any other round.
+//    without barriers, while the others wait.  A loaded graph's rows hold no
+//    head twice, so its decrements are plain loads and stores, SOLO_ILP chunks of
+//    32 arcs in flight; on rows that may (a caller's own, not in increasing
+//    order) they are atomics.  It hands back to the block at any other round.
 //
 // Measured (cycles per round at 1.9 GHz): warp form 2,050 with the arcs in
 // shared memory, 3,200 with the graph's own rows in L2; block form of one
@@ -71,6 +72,7 @@ struct LocalState {
     int nseg;
     long long kD, D, max_rounds;
     int use_min, gpo, lpo;
+    int repeats;         // a row may hold a head more than once
     long long *tr_f_hi;
     unsigned long long *tr_f_lo;
     long long *tr_size, *tr_peeled;
@@ -171,9 +173,10 @@ __device__ __forceinline__ int solo_rounds(const LocalState &S, const Arcs &G, l
                 if (32 * u >= len) break;
                 const int h = cv[u];
                 if (h >= 0) {
-                    const long long nv = tw[h] - cc[u];
-                    if (nv + cc[u] >= 0) {  // live; the row's heads are distinct: no other lane has this one
-                        tw[h] = nv;
+                    long long nv = tw[h] - cc[u];
+                    if (nv + cc[u] >= 0) {  // live
+                        if (S.repeats) nv = (long long)atomicAdd((unsigned long long *)&tw[h], (unsigned long long)(-cc[u])) - cc[u];
+                        else tw[h] = nv;  // the row's heads are distinct: no other lane has this one
                         if (nv < seg[h >> 6]) atomicMin(&seg[h >> 6], nv);
                     }
                 }

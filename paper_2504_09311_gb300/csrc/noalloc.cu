@@ -80,7 +80,9 @@ __global__ void k_noalloc_check(const long long *rp, const int *col, const long 
 
 // ids in range, no self-loops, weights >= 0 (a warp per row; nothing unless the
 // offsets passed, the arc count is even and col is there); flags[4..5] accumulate the symmetry fingerprint (sum over arcs of
-// sym_mix(u, v, c) - sym_mix(v, u, c), zero for a symmetric CSR)
+// sym_mix(u, v, c) - sym_mix(v, u, c), zero for a symmetric CSR); flags[6] = 1
+// when a row is not strictly increasing (it is peeled all the same, but a pair
+// may then stand in it more than once)
 __global__ void k_noalloc_check_arcs(const long long *rp, const int *col, const long long *cw, long long n,
                                      unsigned long long key, int *flags) {
     unsigned long long fp = 0;
@@ -96,6 +98,7 @@ __global__ void k_noalloc_check_arcs(const long long *rp, const int *col, const 
                 atomicExch(&flags[1], 1);
                 continue;
             }
+            if (p > rp[u] && col[p - 1] >= v) atomicExch(&flags[6], 1);
             fp += sym_mix(key, u, v, c) - sym_mix(key, v, u, c);
         }
     }
@@ -149,7 +152,7 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     k_noalloc_check<<<32, 256, 0, s>>>(rp, col, cw, a, n, flags);
     k_noalloc_check_arcs<<<(int)((n + 7) / 8 < 608 ? (n + 7) / 8 : 608), 256, 0, s>>>(rp, col, cw, n, fingerprint_key(), flags);
     DUPIN_CUDA_TRY(cudaGetLastError());
-    int hflags[6] = {0, 0, 0, 0, 0, 0};
+    int hflags[7] = {0, 0, 0, 0, 0, 0, 0};
     DUPIN_CUDA_TRY(cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, s));
     DUPIN_CUDA_TRY(cudaStreamSynchronize(s));
     long long arcs = 0;
@@ -193,6 +196,7 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     A.cl_cap = 0;
     A.one_arcs = 0x7fffffffffffffffLL;
     A.tail_arcs = arcs;
+    A.repeats = hflags[6];
     // the graph itself is the one-CTA kernel's sub-graph (local ids = ids)
     A.tlrp = (long long *)rp;
     A.tcol = (int *)col;

@@ -1242,6 +1242,7 @@ __device__ __forceinline__ void peel_tail_body(const PeelArgs &A, unsigned char 
     S.use_min = A.use_min;
     S.gpo = A.gpo;
     S.lpo = A.lpo;
+    S.repeats = A.repeats;
     S.tr_f_hi = A.tr_f_hi;
     S.tr_f_lo = A.tr_f_lo;
     S.tr_size = A.tr_size;
@@ -1657,6 +1658,7 @@ static PeelArgs make_args(const dupin_graph *g, const PeelWorkspace *ws, const d
     A.cl_c = plan.cl_cap > 0 ? cluster_ctas() : 0;
     A.dmat = ws->tbuf;
     A.again = 0;
+    A.repeats = 0;
     A.tail_smem = 0;
     dense_element(p->metric == DUPIN_DG ? (unsigned long long)DUPIN_Q_ONE : g->w_or, &A.desz, &A.dshift);
     // (without the minimum rule a peel has few rounds, and the dense tail's
