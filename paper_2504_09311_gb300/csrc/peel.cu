@@ -222,8 +222,9 @@ __global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long
 // starts in the tile marks its first arc; a running maximum over the marks gives
 // every arc its row.  Sums are 64-bit differences; a tile with a weight of 2^52
 // or more, whose sums could wrap, first forms the sums of the weights' upper 32
-// bits the same way: a row whose upper sum reaches 2^31 is too heavy, any other
-// cannot wrap.  Bound by issue: four 64-bit finalisers per arc for the
+// bits the same way: a row whose upper sum reaches 2^31 is too heavy, any other's
+// sum is at most 2^63 + 2^43 and cannot wrap; one of 2^63 or more is caught by its
+// sign bit before the vertex weight is added.  Bound by issue: four 64-bit finalisers per arc for the
 // fingerprint.  16.7 million arcs in short rows take 167 us; arcs split evenly
 // over warps with rows found by shuffles took 304 us, and 54 us more for a pass
 // of its own over the weights' signs.
@@ -319,9 +320,10 @@ __global__ void __launch_bounds__(IT_THREADS, 4) k_check_tiles(DevGraph g, long 
                         if (upper) {
                             if (s >= 1LL << 31) bad = true;
                         } else {
+                            if (s < 0) bad = true;
                             s_own[lo - t0] = (int)(r - r0);
                             if (b >= t0 && e <= t1) {
-                                w[r] = s + (g.a ? g.a[r] : 0);  // below 2^64: k_init_reduce sees the sign
+                                w[r] = s + (g.a ? g.a[r] : 0);  // both below 2^63: k_init_reduce sees the sign
                             } else {
                                 const unsigned long long old = atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
                                 if (old + (unsigned long long)s < old) bad = true;
