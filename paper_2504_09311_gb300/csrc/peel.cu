@@ -585,6 +585,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         __syncthreads();
     }
 
+    bool stopped = false;  // max_rounds (the same in every thread)
     for (;;) {
         const long long size = s_st.size;
         // a tail (one CTA or a cluster) takes over once S fits it and either
@@ -597,6 +598,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
             break;
         if (s_st.round >= A.max_rounds) {
             if (b == 0 && tid == 0) set_error(ctl, DUPIN_ERR_NO_PROGRESS);
+            stopped = true;
             break;
         }
         const long long i = s_st.round + 1;
@@ -1051,8 +1053,9 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         }
     }
     // the survivors' weights by id again, for the tails (positions and ids share
-    // w after an even number of compactions, so those pass through w2)
-    if (s_st.size > 0 && s_moved) {
+    // w after an even number of compactions, so those pass through w2); a peel
+    // that stops here has none, and its barriers would fail
+    if (s_st.size > 0 && s_moved && !stopped) {
         const long long L = s_st.live_len;
         const long long j0 = split_at(L, b, G), j1 = split_at(L, b + 1, G);
         const int *live = s_st.live_sel ? A.live1 : A.live0;
