@@ -8,6 +8,7 @@
 // memory, the rounds of local_device.cuh.  Graphs with more than CTA_MAX_N
 // vertices take the single-graph path.  Results are identical to dupin_peel:
 // the arithmetic is the same exact integer peel.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -797,6 +798,29 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
     return DUPIN_OK;
 }
 
+// The end of the page-locked allocation or registration that holds host pointer
+// p, or null where there is none (0.1 us).  The driver's entry point comes through the
+// runtime: the library links no driver.
+static const char *pinned_end(const void *p) {
+    typedef CUresult (*query_t)(void *, CUpointer_attribute, CUdeviceptr);
+    static const query_t query = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (query_t)f;
+    }();
+    CUdeviceptr start = 0;
+    size_t bytes = 0;
+    if (!query || query(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)p) != CUDA_SUCCESS ||
+        query(&bytes, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)p) != CUDA_SUCCESS)
+        return nullptr;
+    return (const char *)start + bytes;
+}
+
 // Copy a finished batch's results into the callers' result structs and free
 // its arena.  'status' gets the first failing graph's code (0 if none).
 int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_status) {
@@ -809,10 +833,14 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
     int status = DUPIN_OK;
     std::string msg;
     if (per_job_status) per_job_status->assign(nj, DUPIN_OK);
-    // peel rounds waiting to be copied: adjacent in the arena and at the caller
+    // Peel rounds waiting to be copied: adjacent in the arena and at the caller,
+    // there inside one page-locked range (the runtime refuses a copy across two,
+    // even where they touch, and what touches in pageable memory may belong to
+    // several callers)
     char *run_to = nullptr;
-    const char *run_from = nullptr;
+    const char *run_from = nullptr, *run_end = nullptr;
     size_t run_bytes = 0;
+    bool run_known = false;  // run_end is the end of run_to's range
     auto flush = [&]() {
         if (run_bytes && e == cudaSuccess) e = cudaMemcpyAsync(run_to, run_from, run_bytes, cudaMemcpyDeviceToHost, s);
         run_bytes = 0;
@@ -846,10 +874,19 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
         const long long n = g->n;
         const int *pr_dev = dev && r.peel_round ? r.peel_round : (const int *)(arena + B->off_pr[k]);
         if (r.peel_round && !dev && n > 0) {
-            if (run_bytes && ((char *)r.peel_round != run_to + run_bytes || (const char *)pr_dev != run_from + run_bytes)) flush();
+            if (run_bytes) {
+                bool joins = (char *)r.peel_round == run_to + run_bytes && (const char *)pr_dev == run_from + run_bytes;
+                if (joins && !run_known) {
+                    run_end = pinned_end(run_to);
+                    run_known = true;
+                }
+                joins = joins && run_end && (const char *)r.peel_round + 4 * (size_t)n <= run_end;
+                if (!joins) flush();
+            }
             if (!run_bytes) {
                 run_to = (char *)r.peel_round;
                 run_from = (const char *)pr_dev;
+                run_known = false;
             }
             run_bytes += 4 * (size_t)n;
         }
