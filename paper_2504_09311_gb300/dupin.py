@@ -436,6 +436,7 @@ def peel_batch(graphs: Sequence[Graph], params: Sequence[Params], want_rounds=Tr
     or a BatchBuffers (reusable: addresses computed once)."""
     k = len(graphs)
     G = np.fromiter((g.handle.value for g in graphs), dtype=np.uint64, count=k)
+    params = list(params)  # any iterable, read twice below
     raw = b"".join(map(bytes, params)) if all(type(p) is Params for p in params) else b""
     # one copy for all of them (the array constructor takes 0.3 us each)
     P = (Params * k).from_buffer_copy(raw) if k and len(raw) == k * ctypes.sizeof(Params) else (Params * k)(*params)
