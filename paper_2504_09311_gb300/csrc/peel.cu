@@ -80,6 +80,49 @@ __global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *li
     }
 }
 
+// Calls fn(r, b, e) once for each row r from r0 on that starts before t1, rows [b,
+// e) of arcs, by any of the block's threads; r0 holds the first arc of the tile that
+// ends at t1 (empty rows may be left out).  A step over NT rows takes about 1 us, and a
+// tile's 2,048 arcs mostly lie in one or two; with far more rows than arcs (ids that
+// were never compacted) the empty ones would take n / 256 steps, 58 ms for 15 million
+// vertices, so after IT_STEPS the rows left are found from the arcs, by a search for
+// each (0.2 ms in all; 8 steps of rows first, 32 and 128 took 20 and 100 us longer).
+#define IT_STEPS 8
+template <int NT, class RowF>
+__device__ __forceinline__ void tile_rows(const DevGraph &g, long long t1, long long r0, RowF fn) {
+    const long long n = g.n;
+    for (int step = 0;; step++) {
+        long long r = r0 + (long long)step * NT + threadIdx.x, b = t1, e = t1;
+        bool end;  // no row further on starts before t1
+        if (step < IT_STEPS) {
+            if (r < n) {
+                b = g.rp[r];
+                e = g.rp[r + 1];
+            }
+            end = r >= n || b >= t1;
+        } else {  // an arc that is the first of its row
+            const long long first = r0 + (long long)IT_STEPS * NT;  // at most n: no earlier step found the end
+            const long long x = g.rp[first] + (long long)(step - IT_STEPS) * NT + threadIdx.x;
+            end = x >= t1;
+            if (!end) {
+                long long lo = first, hi = n - 1;  // the last row that starts at or before x
+                while (lo < hi) {
+                    const long long mid = lo + ((hi - lo + 1) >> 1);
+                    if (g.rp[mid] <= x) lo = mid;
+                    else hi = mid - 1;
+                }
+                if (g.rp[lo] == x) {
+                    r = lo;
+                    b = x;
+                    e = g.rp[lo + 1];
+                }
+            }
+        }
+        if (b < t1) fn(r, b, e);
+        if (__syncthreads_or(end)) return;
+    }
+}
+
 // w_u += sum of c over row u, for peeling: tiles of IT_TILE arc weights
 // arrive in shared memory by bulk copies, two buffers per block; a block scan
 // turns a tile into its running sums (a thread takes eight neighbours, reading
@@ -561,6 +604,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         s_moved = 0;
         s_rd.U_sel = kMaxLL;  // no round yet
         s_rd.arcs = kMaxLL;
+        s_rd.compact = 0;
     }
     __syncthreads();
     if (ctl->status != ST_RUNNING || ctl->error) return;
@@ -585,7 +629,6 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         __syncthreads();
     }
 
-    bool stopped = false;  // max_rounds (the same in every thread)
     for (;;) {
         const long long size = s_st.size;
         // a tail (one CTA or a cluster) takes over once S fits it and either
@@ -597,8 +640,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         if (size == 0 || (size <= A.hcap && s_st.live_len == size && (2 * s_elive <= A.tail_arcs || (small_round && 2 * s_elive <= A.tarc_cap))))
             break;
         if (s_st.round >= A.max_rounds) {
-            if (b == 0 && tid == 0) set_error(ctl, DUPIN_ERR_NO_PROGRESS);
-            stopped = true;
+            s_rd.compact = -1;  // the error is set at the end: it would fail the barrier on the way there
             break;
         }
         const long long i = s_st.round + 1;
@@ -1053,9 +1095,8 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         }
     }
     // the survivors' weights by id again, for the tails (positions and ids share
-    // w after an even number of compactions, so those pass through w2); a peel
-    // that stops here has none, and its barriers would fail
-    if (s_st.size > 0 && s_moved && !stopped) {
+    // w after an even number of compactions, so those pass through w2)
+    if (s_st.size > 0 && s_moved) {
         const long long L = s_st.live_len;
         const long long j0 = split_at(L, b, G), j1 = split_at(L, b + 1, G);
         const int *live = s_st.live_sel ? A.live1 : A.live0;
@@ -1085,6 +1126,7 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         ctl->scan_volume = st.scan;
         if (!ctl->handed) ctl->bulk_rounds = st.round;
         ctl->elive = s_elive;
+        if (s_rd.compact < 0) set_error(ctl, DUPIN_ERR_NO_PROGRESS);
         if (ctl->error == 0)
             ctl->status = st.size == 0 ? ST_DONE : tail_status(A, st.size, 2 * s_elive);
     }
