@@ -86,40 +86,36 @@ __global__ void k_init_vertex(DevGraph g, int dg, long long *w, int *pr, int *li
 // tile's 2,048 arcs mostly lie in one or two; with far more rows than arcs (ids that
 // were never compacted) the empty ones would take n / 256 steps, 58 ms for 15 million
 // vertices, so after IT_STEPS the rows left are found from the arcs, by a search for
-// each (0.2 ms in all; 8 steps of rows first, 32 and 128 took 20 and 100 us longer).
+// each (0.15 ms in all; 32 and 128 steps of rows first took 20 and 100 us longer).
+// (Both forms in one loop: 1.34 ms for 1.29 on R-MAT scale 24.)
 #define IT_STEPS 8
 template <int NT, class RowF>
 __device__ __forceinline__ void tile_rows(const DevGraph &g, long long t1, long long r0, RowF fn) {
+    const int tid = threadIdx.x;
     const long long n = g.n;
-    for (int step = 0;; step++) {
-        long long r = r0 + (long long)step * NT + threadIdx.x, b = t1, e = t1;
-        bool end;  // no row further on starts before t1
-        if (step < IT_STEPS) {
-            if (r < n) {
-                b = g.rp[r];
-                e = g.rp[r + 1];
-            }
-            end = r >= n || b >= t1;
-        } else {  // an arc that is the first of its row
-            const long long first = r0 + (long long)IT_STEPS * NT;  // at most n: no earlier step found the end
-            const long long x = g.rp[first] + (long long)(step - IT_STEPS) * NT + threadIdx.x;
-            end = x >= t1;
-            if (!end) {
-                long long lo = first, hi = n - 1;  // the last row that starts at or before x
-                while (lo < hi) {
-                    const long long mid = lo + ((hi - lo + 1) >> 1);
-                    if (g.rp[mid] <= x) lo = mid;
-                    else hi = mid - 1;
-                }
-                if (g.rp[lo] == x) {
-                    r = lo;
-                    b = x;
-                    e = g.rp[lo + 1];
-                }
-            }
+    long long rb = r0;
+    for (int step = 0; step < IT_STEPS; step++, rb += NT) {
+        const long long r = rb + tid;
+        long long b = t1, e = t1;
+        if (r < n) {
+            b = g.rp[r];
+            e = g.rp[r + 1];
         }
         if (b < t1) fn(r, b, e);
-        if (__syncthreads_or(end)) return;
+        if (__syncthreads_or(r >= n || b >= t1)) return;
+    }
+    // rows rb .. n - 1 (rb <= n): the arcs that are the first of their row
+    for (long long x = g.rp[rb] + tid;; x += NT) {
+        if (x < t1) {
+            long long lo = rb, hi = n - 1;  // the last row that starts at or before x
+            while (lo < hi) {
+                const long long mid = lo + ((hi - lo + 1) >> 1);
+                if (g.rp[mid] <= x) lo = mid;
+                else hi = mid - 1;
+            }
+            if (g.rp[lo] == x) fn(lo, x, g.rp[lo + 1]);
+        }
+        if (__syncthreads_or(x >= t1)) return;
     }
 }
 
@@ -231,24 +227,15 @@ __global__ void __launch_bounds__(IT_THREADS) k_init_tiles(DevGraph g, long long
         __syncthreads();
         // rows that start before the tile's end, from the one holding its first arc on
         const long long t1 = t0 + len;
-        for (long long rb = r0;; rb += IT_THREADS) {
-            const long long r = rb + tid;
-            long long b = t1, e = t1;
-            if (r < n) {
-                b = g.rp[r];
-                e = g.rp[r + 1];
+        tile_rows<IT_THREADS>(g, t1, r0, [&](long long r, long long b, long long e) {
+            const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
+            if (hi > lo) {
+                const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
+                if (b >= t0 && e <= t1) w[r] = s + (g.a ? g.a[r] : 0);
+                else atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
             }
-            if (b < t1) {
-                const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
-                if (hi > lo) {
-                    const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
-                    if (b >= t0 && e <= t1) w[r] = s + (g.a ? g.a[r] : 0);
-                    else atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
-                }
-                if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
-            }
-            if (__syncthreads_or(r >= n || b >= t1)) break;
-        }
+            if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
+        });
         r0 = s_row;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // reads and writes of P before the next copy into it
         __syncthreads();
@@ -349,34 +336,25 @@ __global__ void __launch_bounds__(IT_THREADS, 4) k_check_tiles(DevGraph g, long 
             }
             __syncthreads();
             // rows that start before the tile's end, from the one holding its first arc on
-            for (long long rb = r0;; rb += IT_THREADS) {
-                const long long r = rb + tid;
-                long long b = t1, e = t1;
-                if (r < n) {
-                    b = g.rp[r];
-                    e = g.rp[r + 1];
-                }
-                if (b < t1) {
-                    const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
-                    if (hi > lo) {
-                        const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
-                        if (upper) {
-                            if (s >= 1LL << 31) bad = true;
+            tile_rows<IT_THREADS>(g, t1, r0, [&](long long r, long long b, long long e) {
+                const long long lo = b > t0 ? b : t0, hi = e < t1 ? e : t1;
+                if (hi > lo) {
+                    const long long s = (hi == t1 ? total : P[hi - t0]) - P[lo - t0];
+                    if (upper) {
+                        if (s >= 1LL << 31) bad = true;
+                    } else {
+                        if (s < 0) bad = true;
+                        s_own[lo - t0] = (int)(r - r0);
+                        if (b >= t0 && e <= t1) {
+                            w[r] = s + (g.a ? g.a[r] : 0);  // both below 2^63: k_init_reduce sees the sign
                         } else {
-                            if (s < 0) bad = true;
-                            s_own[lo - t0] = (int)(r - r0);
-                            if (b >= t0 && e <= t1) {
-                                w[r] = s + (g.a ? g.a[r] : 0);  // both below 2^63: k_init_reduce sees the sign
-                            } else {
-                                const unsigned long long old = atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
-                                if (old + (unsigned long long)s < old) bad = true;
-                            }
+                            const unsigned long long old = atomicAdd((unsigned long long *)&w[r], (unsigned long long)s);
+                            if (old + (unsigned long long)s < old) bad = true;
                         }
                     }
-                    if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
                 }
-                if (__syncthreads_or(r >= n || b >= t1)) break;
-            }
+                if (e >= t1) s_row = r;  // at most one row with arcs reaches t1; it, or the next, is first in the next tile
+            });
         }
         // the row of every arc, and its checks
         int own[IT_ITEMS], col[IT_ITEMS];
