@@ -17,10 +17,11 @@
 //
 //  - Warp form, for the minimum-rule rounds of one vertex that make up most of
 //    a weighted peel with k(1+eps) < 2: warp 0 runs round after round alone,
-//    without barriers, while the others wait.  A loaded graph's rows hold no
-//    head twice, so its decrements are plain loads and stores, SOLO_ILP chunks of
-//    32 arcs in flight; on rows that may (a caller's own, not in increasing
-//    order) they are atomics.  It hands back to the block at any other round.
+//    without barriers, while the others wait.  Its decrements are plain loads
+//    and stores, SOLO_ILP chunks of 32 arcs in flight, so no row may hold a head
+//    twice: rows that are not known to be strictly increasing (a caller's own) stay
+//    with the block form and its atomics.  It hands back to the block at any
+//    other round.
 //
 // Measured (cycles per round at 1.9 GHz): warp form 2,050 with the arcs in
 // shared memory, 3,200 with the graph's own rows in L2; block form of one
@@ -32,12 +33,19 @@
 
 #define SOLO_ILP 4                   // 32-arc chunks in flight
 #define SOLO_ARCS (32 * SOLO_ILP)    // most arcs of a warp-form round
-#define SOLO_TRY 2                   // the warp form is tried after this many block-form rounds of one vertex
+#define SOLO_TRY 2                   // the warp form is tried after this many block-form rounds of one vertex ...
+#define SOLO_PAYS 2                  // ... or twice as many as last time, up to SOLO_REST, when it ran fewer
+#define SOLO_REST 64                 // rounds than this: a try costs about 1 us (a core with rows of 160 arcs,
+                                     // which the warp cannot take: 8.3 ms with a try every second round, 6.8 without)
 
 // Where the sub-graph's arcs are.  LocalArcs: copied out, rows end to end, only
 // live heads.  GraphArcs: the whole graph's rows, heads looked up in a map from
 // vertex to local id (negative: gone before the sub-graph was taken).
 struct LocalArcs {
+    // Most segments the warp form looks over (twice a round, alone): with the arcs
+    // at hand a weighted block graph's peel takes 1.15 ms with and 1.09 without it at
+    // 92 segments, 2.62 and 2.43 at 230; 0.63 and 0.70 at 24.
+    static constexpr int kSoloSegs = 64;
     const int *toff;       // [L + 1] first arc of each row, in shared memory
     const int *col;        // local heads ...
     const long long *cw;   // ... and weights (nullptr: 1.0)
@@ -51,6 +59,9 @@ struct LocalArcs {
 };
 
 struct GraphArcs {
+    // (the block's rounds wait twice as long for the graph's rows: 160 windows of
+    // 60,000 edges take 2.59 ms with and 2.69 without the warp form above 64 segments)
+    static constexpr int kSoloSegs = 0x7fffffff;
     const unsigned *start, *deg;  // [L] each row's first arc and arcs, in shared memory
     const int *col, *hubs;
     const long long *cw;          // nullptr: 1.0
@@ -72,7 +83,7 @@ struct LocalState {
     int nseg;
     long long kD, D, max_rounds;
     int use_min, gpo, lpo;
-    int repeats;         // a row may hold a head more than once
+    int repeats;         // a row may hold a head more than once: no warp form
     long long *tr_f_hi;
     unsigned long long *tr_f_lo;
     long long *tr_size, *tr_peeled;
@@ -173,10 +184,9 @@ __device__ __forceinline__ int solo_rounds(const LocalState &S, const Arcs &G, l
                 if (32 * u >= len) break;
                 const int h = cv[u];
                 if (h >= 0) {
-                    long long nv = tw[h] - cc[u];
-                    if (nv + cc[u] >= 0) {  // live
-                        if (S.repeats) nv = (long long)atomicAdd((unsigned long long *)&tw[h], (unsigned long long)(-cc[u])) - cc[u];
-                        else tw[h] = nv;  // the row's heads are distinct: no other lane has this one
+                    const long long nv = tw[h] - cc[u];
+                    if (nv + cc[u] >= 0) {  // live; the row's heads are distinct: no other lane has this one
+                        tw[h] = nv;
                         if (nv < seg[h >> 6]) atomicMin(&seg[h >> 6], nv);
                     }
                 }
@@ -241,10 +251,11 @@ __device__ __forceinline__ int local_rounds(const LocalState &S, const Arcs &G, 
     unsigned short *tf = S.tf;
     long long mins_all = seg_global_min(segbuf + ((st.round + 1) & 1) * nseg, nseg);
     TailRound R = tail_plan<NARROW>(S.kD, S.D, S.use_min, S.gpo, S.lpo, st, mins_all);
-    int ones = 0;  // block-form rounds of one vertex in a row
+    // block-form rounds of one vertex in a row; how many before a try of the warp form
+    int ones = 0, need = S.repeats || nseg > Arcs::kSoloSegs ? 0x7fffffff : SOLO_TRY;
     while (!R.done) {
         if (R.i > S.max_rounds) return DUPIN_ERR_NO_PROGRESS;
-        if (ones >= SOLO_TRY) {
+        if (ones >= need && R.minrule) {
             ones = 0;
             const int b0 = (int)(R.i & 1);
             if (tid == (NW - 1) * 32) {
@@ -294,6 +305,7 @@ __device__ __forceinline__ int local_rounds(const LocalState &S, const Arcs &G, 
             st.best_size = s_hand->best_size;
             st.bf = mk128(s_hand->bf_lo, s_hand->bf_hi);
             mins_all = s_hand->mins;
+            need = s_hand->rounds >= SOLO_PAYS ? SOLO_TRY : need < SOLO_REST ? 2 * need : SOLO_REST;
             const bool odd = s_hand->rounds & 1;  // the minima move to the next round's buffer
             if (odd)
                 for (int q = tid; q < nseg; q += NT) segbuf[(b0 ^ 1) * nseg + q] = segbuf[b0 * nseg + q];
