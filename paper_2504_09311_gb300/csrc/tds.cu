@@ -29,13 +29,13 @@
 // matrix in shared memory, so no clique is visited one by one and w is
 // updated once per (u, v).  Whether two candidates are adjacent comes from one
 // bit of a global matrix over the (at most) CORE_MAX vertices of highest
-// degree, or from a binary search in the row of the one outside it, a short
-// row.  (A row merge or a leapfrog walk per arc, one warp per u, read hub
+// degree; outside it the rows themselves are read, or searched where they are
+// long.  (A row merge or a leapfrog walk per arc, one warp per u, read hub
 // rows of thousands for every arc of a hub.  One peel, k = q: R-MAT scale 15
-// TDS 63.4 -> 1.57 ms, scale 13 4-cliques 417 -> 0.90 ms; what is left is bound
-// by the latency of the bit lookups and row searches, 64 warps per SM.)
-// A warp takes a vertex of at most WARP_P candidates, a CTA one of up to
-// CTA_P (one SM's shared memory; for triangles, which need no matrix, P
+// TDS 63.4 -> 1.32 ms, scale 13 4-cliques 417 -> 0.87 ms; what is left is bound
+// by the latency of the bit lookups and row reads.)
+// A warp takes a vertex of at most WARP_P candidates and LONG_ROW arcs, a CTA one of up to
+// CTA_P candidates (one SM's shared memory; for triangles, which need no matrix, P
 // itself is the limit); larger ones fall back to a depth-first walk over the
 // rows.  Rows are sorted (the loader checks it).
 #include <cuda_runtime.h>
@@ -43,6 +43,7 @@
 
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "dupin_internal.h"
 
@@ -54,12 +55,20 @@ constexpr int CORE_WORDS = CORE_MAX / 32;  // its row
 constexpr int DEG_BINS = 4096;
 constexpr int WARP_P = 128;                // candidates of a warp's vertex
 constexpr int WARP_STRIDE = WARP_P / 32 + 1;
+constexpr int LONG_ROW = 4096;             // a warp reads no longer row for a vertex's candidates
+constexpr int READ_ARCS = 192;             // a candidate's row is read when it has no more arcs than this for every
+                                           // 32 candidates: one step of 32 searches costs as much as six of 32 reads
+constexpr int SEARCHED = -1, READ = -2;    // what happens to the row of a candidate outside the matrix
+constexpr int ROW_ILP = 4;                 // arcs of those rows in flight per thread
+constexpr int WARP_SIEVE = 256, CTA_SIEVE = 1024;  // words of the candidate filter
+constexpr int CTA_ROWS = 4;                // rows a warp of a CTA takes at a time
 constexpr int CTA_P = 1216;                // candidates of a CTA's vertex with a matrix ...
 constexpr int CTA_P3 = 24576;              // ... and without (triangles)
-constexpr int WARP_TEAM = 256, CTA_TEAM = 512;
-constexpr size_t CTA_SMEM = 2 * 4 * CTA_P + 4 * (size_t)CTA_P * (CTA_P / 32 + 1);
+constexpr int WARP_TEAM = 256, CTA_TEAM = 512, CTA_TEAM3 = 1024;  // threads (CTA_TEAM3: triangles)
+constexpr size_t CTA_LISTS = 2 * 4 * CTA_P + 4 * (size_t)CTA_P * (CTA_P / 32 + 1);
+constexpr size_t CTA_SMEM = CTA_LISTS + 4 * CTA_SIEVE;
 static_assert((CTA_P / 32 + 1) % 2 == 1 && WARP_STRIDE % 2 == 1, "an odd row stride spreads rows over the banks");
-static_assert(2 * 4 * (size_t)CTA_P3 <= CTA_SMEM, "triangles' candidates fit the same shared memory");
+static_assert(2 * 4 * (size_t)CTA_P3 <= CTA_LISTS, "triangles' candidates fit the same shared memory");
 
 struct TdsCtl {
     long long round, size, best_round, best_size, n_min_rule;
@@ -303,13 +312,89 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x)
     return (unsigned long long)__shfl_sync(0xffffffffu, warp_sum64((long long)x), 0);
 }
 
-// u's cliques by one warp; false when it has more than WARP_P candidates.
-// Adds the sum over v of the cliques through v, (q-1) times u's, to 'sum'.
+// Pairs of candidates are found in two ways.  Between two members of the adjacency
+// matrix a bit tells, and a long row is searched for the other's id; but a row
+// outside the matrix that is short against the number of candidates is read, and each
+// neighbour looked up among the candidates: in a filter by its id's low bits,
+// then by a search of their ids (increasing, as the row they come from).
+// (TDS, k = 3.  Searches alone took 54 ms on a uniform graph of 300,000 vertices and
+// degree 120, 18.7 ms on 1,000,000 of degree 32 and 146 ms on 50,000 of degree 400, where
+// merging rows had taken 15.6, 7.2 and 28; with the reads it is 15.1, 5.4 and 34.)
+
+// of each candidate outside the matrix: is its row read?  (returns whether this
+// thread found such a one)
+__device__ __forceinline__ bool pick_rows(const TdsArgs &A, const int *ids, int *cis, int p, int t, int nt) {
+    const long long most = (long long)READ_ARCS * ((p + 31) >> 5);
+    bool any = false;
+    for (int v = t; v < p; v += nt) {
+        if (cis[v] >= 0) continue;
+        const bool read = A.rp[ids[v] + 1] - A.rp[ids[v]] <= most;
+        cis[v] = read ? READ : SEARCHED;
+        any = any || read;
+    }
+    return any;
+}
+
+__device__ __forceinline__ unsigned sieve_bit(int x) { return 1u << (x & 31); }
+template <int WORDS>
+__device__ __forceinline__ int sieve_word(int x) { return (x >> 5) & (WORDS - 1); }
+
+// One warp: the rows to be read among candidates g0 .. g0 + per - 1 (per <= 32), their
+// arcs spread over the lanes; hit(v, j) for each neighbour of candidate v that is
+// candidate j.
+template <int WORDS, class Hit>
+__device__ __forceinline__ void read_rows(const TdsArgs &A, const int *ids, const int *cis, int p, const unsigned *sieve,
+                                          int g0, int per, Hit hit) {
+    const int lane = threadIdx.x & 31;
+    const int v = g0 + lane;
+    const bool mine = lane < per && v < p && cis[v] == READ;
+    const long long start = mine ? A.rp[ids[v]] : 0;
+    const int deg = mine ? (int)(A.rp[ids[v] + 1] - start) : 0;
+    int before = deg;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, before, d);
+        if (lane >= d) before += o;
+    }
+    const int all = __shfl_sync(0xffffffffu, before, 31);
+    before -= deg;
+    for (int k0 = lane; k0 - lane < all; k0 += 32 * ROW_ILP) {
+        int t[ROW_ILP], y[ROW_ILP];
+#pragma unroll
+        for (int z = 0; z < ROW_ILP; z++) {
+            const int k = k0 + 32 * z;
+            t[z] = 0;  // the row of arc k: the last that starts at or before it
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, before, t[z] + step) <= k) t[z] += step;
+            const long long at = __shfl_sync(0xffffffffu, start, t[z]) + (k - __shfl_sync(0xffffffffu, before, t[z]));
+            y[z] = k < all ? A.col[at] : 0;
+        }
+#pragma unroll
+        for (int z = 0; z < ROW_ILP; z++) {
+            if (k0 + 32 * z >= all) continue;
+            if (y[z] < 0) y[z] = A.hubs[-y[z] - 1];
+            if (!(sieve[sieve_word<WORDS>(y[z])] & sieve_bit(y[z]))) continue;
+            int lo = 0, hi = p - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (ids[mid] <= y[z]) lo = mid;
+                else hi = mid - 1;
+            }
+            if (ids[lo] == y[z]) hit(g0 + t[z], lo);
+        }
+    }
+}
+
+// u's cliques by one warp; false when it has more than WARP_P candidates or too
+// long a row.  Adds the sum over v of the cliques through v, (q-1) times u's, to 'sum'.
+template <bool TRIANGLES, bool READS>
 __device__ __forceinline__ bool warp_vertex(const TdsArgs &A, int u, int r, int *ids, int *cis, unsigned *rows,
-                                            unsigned long long &sum) {
+                                            unsigned *sieve, unsigned long long &sum) {
     const int lane = threadIdx.x & 31;
     const Keep keep(A, u, r);
     const long long b = A.rp[u], e = A.rp[u + 1];
+    if (e - b > LONG_ROW) return false;
     int p = 0;
     for (long long j0 = b; j0 < e; j0 += 32) {
         const long long j = j0 + lane;
@@ -324,34 +409,57 @@ __device__ __forceinline__ bool warp_vertex(const TdsArgs &A, int u, int r, int 
         }
         p += __popc(bal);
     }
-    const int q = A.q;
+    const int q = TRIANGLES ? 3 : A.q;
     if (p < q - 1) return true;
     __syncwarp();
+    const bool reads = READS && __any_sync(0xffffffffu, pick_rows(A, ids, cis, p, lane, 32));
     const int words = (p + 31) >> 5;
-    unsigned long long mine = 0;
-    for (int v = 0; v < p; v++) {
-        const int x = ids[v], cx = cis[v];
-        int t = 0;
-        for (int w = 0; w < words; w++) {
-            const int y = 32 * w + lane;
-            const unsigned bal = __ballot_sync(0xffffffffu, y < p && y != v && adjacent(A, x, cx, ids[y], cis[y]));
-            if (q == 3) t += __popc(bal);
-            else if (lane == 0) rows[v * WARP_STRIDE + w] = bal;
-        }
-        if (q == 3 && lane == 0) {
-            credit(A, x, (unsigned long long)t, r);
-            mine += (unsigned long long)t;
+    const int stride = TRIANGLES ? 1 : WARP_STRIDE;  // triangles: a count per candidate in place of its matrix row
+    if (reads) {
+        for (int k = lane; k < WARP_SIEVE; k += 32) sieve[k] = 0;
+        for (int k = lane; k < p * stride; k += 32) rows[k] = 0;
+        __syncwarp();
+        for (int v = lane; v < p; v += 32) atomicOr(&sieve[sieve_word<WARP_SIEVE>(ids[v])], sieve_bit(ids[v]));
+    }
+    __syncwarp();
+    // pairs of candidates whose rows are not read
+    for (int g0 = 0; g0 < p; g0 += 32) {
+        unsigned left = __ballot_sync(0xffffffffu, g0 + lane < p && !(READS && cis[g0 + lane] == READ));
+        while (left) {
+            const int v = g0 + __ffs(left) - 1;
+            left &= left - 1;
+            const int x = ids[v], cx = cis[v];
+            int t = 0;
+            for (int w = 0; w < words; w++) {
+                const int y = 32 * w + lane;
+                const bool in = y < p && y != v && !(READS && cis[y] == READ) && adjacent(A, x, cx, ids[y], cis[y]);
+                const unsigned bal = __ballot_sync(0xffffffffu, in);
+                if (TRIANGLES) t += __popc(bal);
+                else if (lane == 0) rows[v * stride + w] = bal;
+            }
+            if (TRIANGLES && lane == 0) rows[v] = t;
         }
     }
     __syncwarp();
-    if (q > 3) {
-        for (int v = lane; v < p; v += 32) {
-            const unsigned long long t = cliques_of(q - 2, rows, WARP_STRIDE, words, v, 0, words);
-            credit(A, ids[v], t, r);
-            mine += t;
-        }
+    for (int g0 = 0; reads && g0 < p; g0 += 32)
+        read_rows<WARP_SIEVE>(A, ids, cis, p, sieve, g0, 32, [&](int v, int j) {
+            const bool both = cis[j] != READ;  // j's row will not tell
+            if (TRIANGLES) {
+                atomicAdd(&rows[v], 1u);
+                if (both) atomicAdd(&rows[j], 1u);
+            } else {
+                atomicOr(&rows[v * stride + (j >> 5)], 1u << (j & 31));
+                if (both) atomicOr(&rows[j * stride + (v >> 5)], 1u << (v & 31));
+            }
+        });
+    __syncwarp();
+    unsigned long long found = 0;
+    for (int v = lane; v < p; v += 32) {
+        const unsigned long long t = TRIANGLES ? rows[v] : cliques_of(q - 2, rows, stride, words, v, 0, words);
+        credit(A, ids[v], t, r);
+        found += t;
     }
-    sum += mine;
+    sum += found;
     __syncwarp();
     return true;
 }
@@ -368,10 +476,11 @@ __device__ __forceinline__ void add_cliques(const TdsArgs &A, unsigned long long
     }
 }
 
-template <bool ROUND>
-__global__ void __launch_bounds__(WARP_TEAM) k_clq_warp(TdsArgs A) {
+template <bool ROUND, bool TRIANGLES, bool READS>
+__global__ void __launch_bounds__(WARP_TEAM, TRIANGLES ? 5 : 3) k_clq_warp(TdsArgs A) {
     __shared__ int s_ids[WARP_TEAM / 32][WARP_P], s_cis[WARP_TEAM / 32][WARP_P];
-    __shared__ unsigned s_rows[WARP_TEAM / 32][WARP_P * WARP_STRIDE];
+    __shared__ unsigned s_rows[WARP_TEAM / 32][TRIANGLES ? WARP_P : WARP_P * WARP_STRIDE];
+    __shared__ unsigned s_sieve[READS ? WARP_TEAM / 32 : 1][WARP_SIEVE];
     const TdsCtl *c = A.ctl;
     if (ROUND && (c->status || c->error)) return;
     const int r = ROUND ? (int)(c->round + 1) : -1;
@@ -382,7 +491,7 @@ __global__ void __launch_bounds__(WARP_TEAM) k_clq_warp(TdsArgs A) {
     for (long long k = blockIdx.x * (long long)(WARP_TEAM / 32) + wid; k < U; k += W) {
         const int u = ROUND ? A.front[k] : (int)k;
         unsigned long long sum = 0;
-        if (!warp_vertex(A, u, r, s_ids[wid], s_cis[wid], s_rows[wid], sum)) {
+        if (!warp_vertex<TRIANGLES, READS>(A, u, r, s_ids[wid], s_cis[wid], s_rows[wid], s_sieve[READS ? wid : 0], sum)) {
             if (lane == 0) A.big[atomicAdd(&A.ctl->nbig, 1)] = u;
             __syncwarp();
             continue;
@@ -494,21 +603,22 @@ __device__ void clique_walk(const TdsArgs &A, int q, int u, long long j, long lo
 
 
 // Vertices with more candidates than a warp takes, a CTA each.
-template <bool ROUND>
-__global__ void __launch_bounds__(CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
+template <bool ROUND, bool TRIANGLES, bool READS>
+__global__ void __launch_bounds__(TRIANGLES ? CTA_TEAM3 : CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
     extern __shared__ int s_mem[];
-    __shared__ int s_cnt[CTA_TEAM / 32];
+    constexpr int TEAM = TRIANGLES ? CTA_TEAM3 : CTA_TEAM;
+    constexpr int NW = TEAM / 32;
+    __shared__ int s_cnt[NW];
     __shared__ unsigned long long s_sum;
-    constexpr int NW = CTA_TEAM / 32;
     const TdsCtl *c = A.ctl;
     if (ROUND && (c->status || c->error)) return;
     const int r = ROUND ? (int)(c->round + 1) : -1;
     const int nbig = c->nbig;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int q = A.q;
-    const int cap = q == 3 ? CTA_P3 : CTA_P;
+    const int q = TRIANGLES ? 3 : A.q;
+    const int cap = TRIANGLES ? CTA_P3 : CTA_P;
     int *ids = s_mem, *cis = s_mem + cap;
-    unsigned *rows = (unsigned *)(cis + cap);
+    unsigned *rows = (unsigned *)(cis + cap), *sieve = (unsigned *)s_mem + CTA_LISTS / 4;
     unsigned long long total = 0;
     for (int k = blockIdx.x; k < nbig; k += gridDim.x) {
         const int u = A.big[k];
@@ -517,7 +627,7 @@ __global__ void __launch_bounds__(CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
         __syncthreads();
         if (tid == 0) s_sum = 0;
         int p = 0;
-        for (long long j0 = b; j0 < e && p <= cap; j0 += CTA_TEAM) {  // candidates in id order
+        for (long long j0 = b; j0 < e && p <= cap; j0 += TEAM) {  // candidates in id order
             const long long j = j0 + tid;
             const int x = j < e ? head(A, j) : 0;
             const bool kp = j < e && keep(A, x);
@@ -540,7 +650,7 @@ __global__ void __launch_bounds__(CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
         __syncthreads();
         unsigned long long mine = 0;  // this thread's part of the cliques through each candidate
         if (p > cap) {  // too many candidates for shared memory: walk the rows
-            for (long long j = b + tid; j < e; j += CTA_TEAM) {
+            for (long long j = b + tid; j < e; j += TEAM) {
                 const int v = head(A, j);
                 if (!keep(A, v)) continue;
                 clique_walk(A, q, u, j, e, v, [&](int x) { return keep(A, x); }, [&](const int *m) {
@@ -550,22 +660,45 @@ __global__ void __launch_bounds__(CTA_TEAM, 1) k_clq_cta(TdsArgs A) {
             }
         } else if (p >= q - 1) {
             const int words = (p + 31) >> 5, stride = words | 1;
+            const bool reads = READS && __syncthreads_or(pick_rows(A, ids, cis, p, tid, TEAM));
+            if (reads) {
+                for (int w = tid; w < CTA_SIEVE; w += TEAM) sieve[w] = 0;
+                if (!TRIANGLES)
+                    for (int w = tid; w < p * stride; w += TEAM) rows[w] = 0;
+                __syncthreads();
+                for (int v = tid; v < p; v += TEAM) atomicOr(&sieve[sieve_word<CTA_SIEVE>(ids[v])], sieve_bit(ids[v]));
+            }
             for (int v = wid; v < p; v += NW) {
                 const int x = ids[v], cx = cis[v];
+                if (READS && cx == READ) continue;
                 int t = 0;
                 for (int w = 0; w < words; w++) {
                     const int y = 32 * w + lane;
-                    const unsigned bal = __ballot_sync(0xffffffffu, y < p && y != v && adjacent(A, x, cx, ids[y], cis[y]));
-                    if (q == 3) t += __popc(bal);
+                    const unsigned bal = __ballot_sync(
+                        0xffffffffu, y < p && y != v && !(READS && cis[y] == READ) && adjacent(A, x, cx, ids[y], cis[y]));
+                    if (TRIANGLES) t += __popc(bal);
                     else if (lane == 0) rows[(size_t)v * stride + w] = bal;
                 }
-                if (q == 3 && lane == 0) {
+                if (TRIANGLES && lane == 0) {
                     credit(A, x, (unsigned long long)t, r);
                     mine += (unsigned long long)t;
                 }
             }
             __syncthreads();
-            if (q > 3) {
+            for (int g0 = CTA_ROWS * wid; reads && g0 < p; g0 += CTA_ROWS * NW)
+                read_rows<CTA_SIEVE>(A, ids, cis, p, sieve, g0, CTA_ROWS, [&](int v, int j) {
+                    const bool both = cis[j] != READ;  // j's row will not tell
+                    if (TRIANGLES) {
+                        credit(A, ids[v], 1, r);
+                        if (both) credit(A, ids[j], 1, r);
+                        mine += both ? 2 : 1;
+                    } else {
+                        atomicOr(&rows[(size_t)v * stride + (j >> 5)], 1u << (j & 31));
+                        if (both) atomicOr(&rows[(size_t)j * stride + (v >> 5)], 1u << (v & 31));
+                    }
+                });
+            if (reads) __syncthreads();
+            if (!TRIANGLES) {
                 for (int v = wid; v < p; v += NW) {  // lanes share the first member's words
                     unsigned long long t = 0;
                     for (int w = lane; w < words; w += 32) t += cliques_of(q - 2, rows, stride, words, v, w, w + 1);
@@ -720,7 +853,10 @@ int set_clique_smem() {
     if (dev < 0 || dev >= 64) return dupin_fail(DUPIN_ERR_CUDA, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(mu);
     if (done[dev]) return DUPIN_OK;
-    for (const void *f : {(const void *)k_clq_cta<false>, (const void *)k_clq_cta<true>}) {
+    for (const void *f : {(const void *)k_clq_cta<false, false, false>, (const void *)k_clq_cta<true, false, false>,
+                          (const void *)k_clq_cta<false, true, false>, (const void *)k_clq_cta<true, true, false>,
+                          (const void *)k_clq_cta<false, false, true>, (const void *)k_clq_cta<true, false, true>,
+                          (const void *)k_clq_cta<false, true, true>, (const void *)k_clq_cta<true, true, true>}) {
         cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CTA_SMEM);
         if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncSetAttribute(k_clq_cta)");
     }
@@ -788,13 +924,25 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
     const int vgrid = (int)std::max<long long>(1, std::min<long long>(sms * 8, (n + 255) / 256));
     const int cgrid = (int)std::max<long long>(1, std::min<long long>(sms, (n + 1023) / 1024));
     const int wgrid = (int)std::max<long long>(1, std::min<long long>(sms * 8, (n + WARP_TEAM / 32 - 1) / (WARP_TEAM / 32)));
+    // the two listing launches, in the form for this peel: 'round', triangles or
+    // not, rows read or not (up to CORE_MAX vertices all are in the matrix)
+    auto list = [&](auto round, auto triangles, auto reads) {
+        constexpr bool R = decltype(round)::value, T = decltype(triangles)::value, D = decltype(reads)::value;
+        k_clq_warp<R, T, D><<<wgrid, WARP_TEAM, 0, s>>>(A);
+        k_clq_cta<R, T, D><<<sms, T ? CTA_TEAM3 : CTA_TEAM, CTA_SMEM, s>>>(A);
+    };
+    auto listing = [&](auto round) {
+        if (A.q == 3 && n > CORE_MAX) list(round, std::true_type{}, std::true_type{});
+        else if (A.q == 3) list(round, std::true_type{}, std::false_type{});
+        else if (n > CORE_MAX) list(round, std::false_type{}, std::true_type{});
+        else list(round, std::false_type{}, std::false_type{});
+    };
     k_tds_reset<<<vgrid, 256, 0, s>>>(A);
     k_core_hist<<<vgrid, 256, 0, s>>>(A);
     k_core_threshold<<<1, 1024, 0, s>>>(A);
     k_core_rows<<<vgrid, 256, 0, s>>>(A);
     k_core_bits<<<wgrid, WARP_TEAM, 0, s>>>(A);
-    k_clq_warp<false><<<wgrid, WARP_TEAM, 0, s>>>(A);
-    k_clq_cta<false><<<sms, CTA_TEAM, CTA_SMEM, s>>>(A);
+    listing(std::false_type{});
     k_tds_start<<<1, 1, 0, s>>>(A);
     k_tds_close<<<cgrid, 1024, 0, s>>>(A, 1);
     TdsCtl hc;
@@ -802,8 +950,7 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
     for (long long done_rounds = 0;; done_rounds += group, group = group < 32 ? 2 * group : 32) {
         for (int j = 0; j < group; j++) {
             k_tds_select<<<vgrid, 256, 0, s>>>(A);
-            k_clq_warp<true><<<wgrid, WARP_TEAM, 0, s>>>(A);
-            k_clq_cta<true><<<sms, CTA_TEAM, CTA_SMEM, s>>>(A);
+            listing(std::true_type{});
             k_tds_close<<<cgrid, 1024, 0, s>>>(A, 0);
         }
         e = cudaGetLastError();
