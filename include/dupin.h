@@ -135,8 +135,13 @@ int dupin_graph_load(const dupin_graph_desc *desc, void *stream, dupin_graph **o
  */
 int dupin_graph_free(dupin_graph *g);
 
-/* Free the peeling workspaces kept from freed graphs and release the graph
- * memory the library's pool keeps on the current device (see dupin_graph_free). */
+/* Free the peeling workspaces kept from freed graphs and release the memory the
+ * library's pools keep on the current device: that of freed graphs (see
+ * dupin_graph_free), and up to DUPIN_SCRATCH_KEEP bytes of call state
+ * (dupin_peel_batch and the server: the batch's state; dupin_peel under the clique
+ * metrics), which stay for the next such call.  Call state beyond that goes back
+ * to the device by itself. */
+#define DUPIN_SCRATCH_KEEP (1ull << 30)
 int dupin_trim_cache(void);
 
 /* n = vertices, m = undirected edges, arcs = 2m, device_bytes = bytes held. */
@@ -331,7 +336,9 @@ int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32_t *col_idx
 typedef struct dupin_server dupin_server;
 
 typedef struct {
-    int64_t memory_budget; /* device bytes the server may hold for per-request state (> 0) */
+    int64_t memory_budget; /* device bytes the server may hold for per-request state (> 0): that of
+                              the requests on the device; what finished ones leave in the library's
+                              pool (dupin_trim_cache) is not counted */
     int32_t max_slots;     /* requests on the device at once, 1..4096 */
     int32_t device;        /* CUDA device ordinal */
 } dupin_serve_config;

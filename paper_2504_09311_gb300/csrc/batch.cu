@@ -662,7 +662,7 @@ long long cta_job_bytes(const dupin_graph *g, const dupin_params *p) {
 }
 
 struct CtaBatch {
-    unsigned char *arena = nullptr;  // from the graphs' pool, which keeps freed memory
+    unsigned char *arena = nullptr;  // from the scratch pool
     size_t nj = 0, outs_base = 0;
     std::vector<size_t> off_pr, off_tr;
     std::vector<long long> trcap;
@@ -724,7 +724,7 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
         at += 4 * (size_t)graphs[idx[k]]->n;
     }
     at = align256(at);
-    cudaError_t e = graph_pool_alloc((void **)&B->arena, at, s);
+    cudaError_t e = scratch_alloc((void **)&B->arena, at, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete B;
@@ -790,7 +790,7 @@ int cta_batch_enqueue(dupin_graph *const *graphs, const dupin_params *params, du
         e = cudaLaunchKernel(shape.fn, dim3(grid), dim3(shape.threads), args, (size_t)dyn, s);
     }
     if (e != cudaSuccess) {
-        graph_pool_free(B->arena, s);
+        scratch_free(B->arena, s);
         delete B;
         return dupin_cuda_fail(e, "batched peel launch");
     }
@@ -930,7 +930,7 @@ int cta_batch_finish(CtaBatch *B, cudaStream_t s, std::vector<int> *per_job_stat
     }
     flush();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    graph_pool_free(arena, s);
+    scratch_free(arena, s);
     delete B;
     if (e != cudaSuccess) return dupin_cuda_fail(e, "batched peel");
     if (status) return dupin_fail(status, msg);

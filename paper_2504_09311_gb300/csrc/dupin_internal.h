@@ -98,11 +98,11 @@ void workspace_free(PeelWorkspace *ws);
 void workspace_free(PeelWorkspace *ws, cudaStream_t s);
 // a freed graph's workspace: kept for a later graph it fits, or freed
 void workspace_release(PeelWorkspace *ws);
-// release the freed graph buffers the library's memory pool keeps (current device)
-void graph_pool_trim();
-// stream-ordered device memory from that pool
-cudaError_t graph_pool_alloc(void **p, size_t bytes, cudaStream_t s);
-void graph_pool_free(void *p, cudaStream_t s);
+// release the freed memory the library's pools keep (current device)
+void pools_trim();
+// stream-ordered device memory for the state of one call
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);
+void scratch_free(void *p, cudaStream_t s);
 int workspace_ensure(dupin_graph *g, const PeelPlan &plan);
 // workspace k of graph g (0: the one dupin_peel uses), allocated or grown for plan
 PeelWorkspace *workspace_slot(dupin_graph *g, int k, const PeelPlan &plan, int *rc);

@@ -23,17 +23,22 @@
 
 #include <map>
 #include <mutex>
+#include <utility>
 #include "dupin_internal.h"
 
 // Device buffers of graphs come from a memory pool of the library's own,
 // stream-ordered, that keeps freed memory (dupin_trim_cache releases it): a
 // caller that loads a new graph for every peel then pays no cudaMalloc /
-// cudaFree for the adjacency and the loader's temporaries.
-static cudaMemPool_t graph_pool(int dev) {
+// cudaFree for the adjacency and the loader's temporaries.  The state of one call
+// (a batch's arena, a clique peel's) comes from a second one, which keeps no more
+// than DUPIN_SCRATCH_KEEP of it and gives the rest back to the device when a
+// stream is next waited for.
+enum { POOL_GRAPHS, POOL_SCRATCH };
+static cudaMemPool_t device_pool(int dev, int which) {
     static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
+    static std::map<std::pair<int, int>, cudaMemPool_t> pools;
     std::lock_guard<std::mutex> lk(mu);
-    auto it = pools.find(dev);
+    auto it = pools.find({dev, which});
     if (it != pools.end()) return it->second;
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
@@ -46,32 +51,36 @@ static cudaMemPool_t graph_pool(int dev) {
         cudaGetLastError();
         return nullptr;
     }
-    unsigned long long keep = ~0ull;
+    unsigned long long keep = which == POOL_GRAPHS ? ~0ull : DUPIN_SCRATCH_KEEP;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    pools[dev] = pool;
+    pools[{dev, which}] = pool;
     return pool;
 }
 
-static cudaError_t galloc(void **p, size_t bytes, cudaStream_t s) {
+static cudaError_t pool_alloc(int which, void **p, size_t bytes, cudaStream_t s) {
     int dev = 0;
     cudaGetDevice(&dev);
-    cudaMemPool_t pool = graph_pool(dev);
+    cudaMemPool_t pool = device_pool(dev, which);
     if (!bytes) bytes = 8;
     return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
 }
+
+static cudaError_t galloc(void **p, size_t bytes, cudaStream_t s) { return pool_alloc(POOL_GRAPHS, p, bytes, s); }
 
 static void gfree(void *p, cudaStream_t s) {
     if (p) cudaFreeAsync(p, s);
 }
 
-cudaError_t graph_pool_alloc(void **p, size_t bytes, cudaStream_t s) { return galloc(p, bytes, s); }
-void graph_pool_free(void *p, cudaStream_t s) { gfree(p, s); }
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) { return pool_alloc(POOL_SCRATCH, p, bytes, s); }
+void scratch_free(void *p, cudaStream_t s) { gfree(p, s); }
 
-void graph_pool_trim() {
+void pools_trim() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return;
-    cudaMemPool_t pool = graph_pool(dev);
-    if (pool) cudaMemPoolTrimTo(pool, 0);
+    for (int which : {POOL_GRAPHS, POOL_SCRATCH}) {
+        cudaMemPool_t pool = device_pool(dev, which);
+        if (pool) cudaMemPoolTrimTo(pool, 0);
+    }
 }
 
 __global__ void k_add_offset_i64(long long *x, long long n, long long add) {

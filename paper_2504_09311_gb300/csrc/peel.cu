@@ -1602,7 +1602,7 @@ extern "C" int dupin_trim_cache(void) {
         workspace_free(ws);
     }
     cudaSetDevice(dev);
-    graph_pool_trim();
+    pools_trim();
     return DUPIN_OK;
 }
 

@@ -888,8 +888,8 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
     A.tr_cap = tr_cap;
     int rc = set_clique_smem();
     if (rc) return rc;
-    // one block from the graphs' pool (it keeps freed memory; the default pool
-    // would give it back to the driver at every call's end)
+    // one block from the scratch pool (the default pool would give it back to the
+    // driver at every call's end)
     size_t at = 0;
     auto part = [&](size_t bytes) {
         const size_t o = at;
@@ -902,13 +902,13 @@ int tds_peel(dupin_graph *g, const dupin_params *p, dupin_result *r, cudaStream_
                  o_hist = part(4 * DEG_BINS), o_mask = part((size_t)n),
                  o_bits = part(4 * (size_t)CORE_WORDS * (size_t)std::min<long long>(n, CORE_MAX));
     unsigned char *buf = nullptr;
-    cudaError_t e = graph_pool_alloc((void **)&buf, at, s);
+    cudaError_t e = scratch_alloc((void **)&buf, at, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return dupin_fail(e == cudaErrorMemoryAllocation ? DUPIN_ERR_OOM : DUPIN_ERR_CUDA,
                           std::string("clique peel state: ") + cudaGetErrorString(e));
     }
-    auto release = [&]() { graph_pool_free(buf, s); };
+    auto release = [&]() { scratch_free(buf, s); };
     A.w = (long long *)(buf + o_w);
     A.pr = (int *)(buf + o_pr);
     A.front = (int *)(buf + o_front);
