@@ -1396,8 +1396,7 @@ int peel_grid_size() {
 }
 
 // raise k_peel_tail's dynamic shared-memory limit, once per device (the
-// limit is a per-device attribute of the function); every launch takes all of
-// it, for the sub-graph's arcs beside the vertex state
+// limit is a per-device attribute of the function)
 static int set_tail_smem(int *bytes) {
     static std::mutex mu;
     static int done[64] = {0};
@@ -1418,6 +1417,16 @@ static int set_tail_smem(int *bytes) {
     if (e != cudaSuccess) return dupin_cuda_fail(e, "cudaFuncSetAttribute(k_peel_tail)");
     *bytes = done[dev] = dyn;
     return DUPIN_OK;
+}
+
+// A launch's dynamic shared memory: the state of up to 'size' vertices and, as far as
+// they fit, up to 'arcs' arcs beside it.  (All of an SM's would keep a small peel
+// waiting for one that no other kernel uses any of.)
+static int tail_smem(long long size, long long arcs, bool weights, int *bytes) {
+    int most = 0;
+    const int rc = set_tail_smem(&most);
+    *bytes = (int)std::min<long long>(most, local_bytes(size, 4) + std::min<long long>(arcs, most) * (weights ? 12 : 4));
+    return rc;
 }
 
 static int check_params(const dupin_graph *g, const dupin_params *p) {
@@ -1783,7 +1792,7 @@ int enqueue_peel_stages(const dupin_graph *g, PeelWorkspace *ws, const dupin_par
         int rc2;
         if (plan.tail_cap > 0) {
             int dyn = 0;
-            if ((rc2 = set_tail_smem(&dyn))) return rc2;
+            if ((rc2 = tail_smem(std::min(plan.tail_cap, g->n), g->arcs, A.tcw != nullptr, &dyn))) return rc2;
             A.tail_smem = dyn;
             k_peel_tail<<<1, TAIL_THREADS, (size_t)dyn, s>>>(A);
         }
@@ -1929,7 +1938,7 @@ int launch_small_graph_peel(const PeelArgs &A, int metric, bool check, cudaStrea
     k_init_finish<<<1, 1, 0, s>>>(A, A.g.n);
     PeelArgs B = A;
     int dyn = 0;
-    rc = set_tail_smem(&dyn);
+    rc = tail_smem(A.g.n, A.g.arcs, A.tcw != nullptr, &dyn);
     if (rc) return rc;
     B.tail_smem = dyn;
     k_peel_tail<<<1, TAIL_THREADS, (size_t)dyn, s>>>(B);
