@@ -28,16 +28,17 @@ typedef unsigned __int128 u128;
 // takes over after such a round whatever the live arc count.
 #define DUPIN_TAIL_SMALL_ROUND 64
 #define DUPIN_TAIL_SMALL_ARCS (1LL << 18)
-// The one-CTA tail takes a live set of at most tail_cap vertices only when
-// its sub-graph has at most this many arcs (one SM fetches them); larger
-// ones go to the cluster tail.
-#define DUPIN_ONE_CTA_ARCS (1LL << 20)
-// ... and to the dense tail, where it fits, from this many arcs on: its round
-// takes 1.0 us, the one-CTA tail's 1.4 us and up (2.2 us at 830,000 arcs over
-// 5,000 vertices), but its build costs four launches and the matrix
-#define DUPIN_DENSE_ARCS (1LL << 16)
-// ... provided its live sub-graph fits the tail's arc buffer (2^27 arcs)
+// The live sub-graph it hands over fits the tail's arc buffer, of at most this
+// many arcs.
 #define DUPIN_TAIL_BUF_ARCS (1LL << 27)
+// The one-CTA tail takes a live set of at most tail_cap vertices only when
+// its sub-graph has at most DUPIN_ONE_CTA_ARCS arcs (one SM fetches them); larger
+// ones go to the cluster tail.  Where the dense tail's matrix fits, it takes the
+// live set from DUPIN_DENSE_ARCS arcs on: its round takes 1.0 us, the one-CTA
+// tail's 1.4 us and up (2.1 us at 840,000 arcs over 5,000 vertices), but its build
+// costs four launches and the matrix.
+#define DUPIN_ONE_CTA_ARCS (1LL << 20)
+#define DUPIN_DENSE_ARCS (1LL << 16)
 // On graphs of at least this many arcs the cluster tail gives the peel back to
 // the grid-wide rounds when the live set collapses: a threshold round of this
 // many vertices, with another threshold round to follow.  (R-MAT scale 24, FD:
@@ -76,7 +77,8 @@ struct PeelCtl {
     long long n_min_rule;
     long long scan_volume;
     long long bulk_rounds;
-    long long elive;      // |E(S)|: undirected edges with both ends live
+    long long elive;      // |E(S)|: undirected edges with both ends live (an upper bound once a
+                          // cluster tail gave the peel back: its own rounds do not count them)
     long long tail_arcs;  // arcs of the tail sub-graph (0 if the tail did not run)
     unsigned long long init_lo, init_hi;  // sum over u of (w_u + a_u) = 2 f(V)
     long long init_min;

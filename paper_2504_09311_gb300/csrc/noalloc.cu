@@ -63,8 +63,7 @@ int scratch_address(int dev, unsigned char **out) {
 
 // flags[0] = 1 when an offset or vertex weight is out of range (flags[1]: an id
 // or arc weight, set by the second check); flags[2..3] = rp[n]
-__global__ void k_noalloc_check(const long long *rp, const int *col, const long long *cw, const long long *a,
-                                long long n, int *flags) {
+__global__ void k_noalloc_check(const long long *rp, const long long *a, long long n, int *flags) {
     for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x) {
         const long long b = rp[u], e = rp[u + 1];
         if (b > e || (u == 0 && b != 0)) {
@@ -74,8 +73,6 @@ __global__ void k_noalloc_check(const long long *rp, const int *col, const long 
         if (a && a[u] < 0) atomicExch(&flags[0], 1);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *(long long *)(flags + 2) = rp[n];
-    (void)col;
-    (void)cw;
 }
 
 // ids in range, no self-loops, weights >= 0 (a warp per row; nothing unless the
@@ -149,7 +146,7 @@ extern "C" int dupin_peel_noalloc(int64_t n, const int64_t *row_ptr, const int32
     // launches and waits: 283 us with a wait after each check and after the
     // mask, and with grids for large graphs; 192 us with two waits and grids
     // of the graph's size (one wait less: 35 us)
-    k_noalloc_check<<<32, 256, 0, s>>>(rp, col, cw, a, n, flags);
+    k_noalloc_check<<<32, 256, 0, s>>>(rp, a, n, flags);
     k_noalloc_check_arcs<<<(int)((n + 7) / 8 < 608 ? (n + 7) / 8 : 608), 256, 0, s>>>(rp, col, cw, n, fingerprint_key(), flags);
     DUPIN_CUDA_TRY(cudaGetLastError());
     int hflags[7] = {0, 0, 0, 0, 0, 0, 0};

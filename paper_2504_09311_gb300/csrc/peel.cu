@@ -614,7 +614,9 @@ __device__ __forceinline__ void peel_bulk_body(const PeelArgs &A, const int b, c
         // vertices or arcs costs a tail microseconds and the grid-wide kernel
         // its barriers)
         const bool small_round = s_rd.U_sel <= DUPIN_TAIL_SMALL_ROUND || s_rd.arcs <= DUPIN_TAIL_SMALL_ARCS;
-        // (and the live list holds nobody else)
+        // (and the live list holds nobody else).  In a peel that was given back, |E(S)| is
+        // the first hand-over's less what has left since: never too small for the
+        // buffer, and the small rounds end the stage.
         if (size == 0 || (size <= A.hcap && s_st.live_len == size && (2 * s_elive <= A.tail_arcs || (small_round && 2 * s_elive <= A.tarc_cap))))
             break;
         if (s_st.round >= A.max_rounds) {
